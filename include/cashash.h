@@ -203,10 +203,10 @@ void cashash_plan_destroy(cashash_plan* plan);
  * match_off is still complete, nothing beyond cap is written and
  * cashash_sync_status() returns EOVERFLOW.  Asynchronous on `stream`.
  * With the persistent schedule all pairs are matched by one batched kernel:
- * by default a bucket join whose Hamming distances come from the tensor cores
- * when every query image fits its shared-memory counters (at least 40,000
- * features), else a speculative per-query kernel (cashash_plan_autotune may
- * choose otherwise); the launch sequence
+ * by default a bucket join when every query image has at most about 50,000
+ * features (at least 40,000 whatever the parameters), else a speculative
+ * per-query kernel (cashash_plan_autotune may choose otherwise); the launch
+ * sequence
  * is captured once as a CUDA graph (per set of output pointers, F and
  * profiling setting) and replayed on `stream`; calls on the same plan must
  * not overlap.
@@ -228,8 +228,8 @@ int cashash_plan_set_threshold_hint(cashash_plan* plan, uint32_t hamming, int fi
  * counterpart (it runs one kernel shape). */
 enum { CASHASH_KERNEL_JOIN = 1, CASHASH_KERNEL_QUERY = 2, CASHASH_KERNEL_JOIN_TC = 3, CASHASH_KERNEL_WARP = 4 };
 typedef struct {
-  uint32_t kernel;       /* CASHASH_KERNEL_JOIN: bucket join with warp-level (mma.sync) tensor-core
-                            Hamming distances (query images that fit its shared-memory counters);
+  uint32_t kernel;       /* CASHASH_KERNEL_JOIN: bucket join, one query per lane (query images of up
+                            to at least 40,000 features);
                             CASHASH_KERNEL_JOIN_TC: the same join with tcgen05 MMAs into tensor
                             memory, 128 query rows per tile (same limit);
                             CASHASH_KERNEL_QUERY: per-query speculative kernel over shared-memory
@@ -237,8 +237,7 @@ typedef struct {
                             CASHASH_KERNEL_WARP: one warp per query, exact without a threshold guess
                             (no calibration; the fit for a few pairs, where the other kernels leave
                             most SMs idle) */
-  uint32_t tile;         /* JOIN: candidate tiles of 8 columns held in registers (2 or 4; 4 with
-                            the band); JOIN_TC, WARP: ignored (0);
+  uint32_t tile;         /* JOIN: 2 or 4 (4 with the band), without effect; JOIN_TC, WARP: ignored (0);
                             QUERY: queries per CTA (256, or 512 when top_k <= 16) */
   uint32_t ctas_per_sm;  /* JOIN, JOIN_TC: resident CTAs per SM, 0 = as many as fit (JOIN_TC: at most
                             2); QUERY, WARP: ignored */

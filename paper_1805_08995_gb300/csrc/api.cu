@@ -709,8 +709,8 @@ int plan_configure(cashash_plan* pl, cashash_tuning t) {
     t = cashash_tuning{};
   } else if (t.kernel == CASHASH_KERNEL_JOIN || t.kernel == CASHASH_KERNEL_JOIN_TC) {
     if (t.kernel == CASHASH_KERNEL_JOIN) {
-      t.tile = (t.tile <= 2 && !epi) ? 2u : 4u;  // the band form has 4 candidate tiles only
-      grid = join_grid(c->kp, pl->na_max, P, t.tile, t.ctas_per_sm);
+      t.tile = (t.tile <= 2 && !epi) ? 2u : 4u;  // (no effect)
+      grid = join_grid(c->kp, pl->na_max, P, t.ctas_per_sm);
     } else {
       t.tile = 0;
       t.ctas_per_sm = t.ctas_per_sm > 2 ? 0u : t.ctas_per_sm;
@@ -935,7 +935,7 @@ int enqueue_match(cashash_ctx* c, cashash_plan* pl, const double* F_dev, uint64_
     if (!warp_only) {
       StageTimer tm(c, CASHASH_STAGE_MATCH, stream, capturing);
       if (pl->join && pl->tune.kernel == CASHASH_KERNEL_JOIN_TC) CK(launch_join_tc(a, pl->grid, stream));
-      else if (pl->join) CK(launch_join(a, pl->grid, pl->tune.tile, stream));
+      else if (pl->join) CK(launch_join(a, pl->grid, stream));
       else CK(launch_match(a, 1, pl->grid, stream, pl->tune.tile));
     }
     {
@@ -1116,14 +1116,13 @@ int cashash_plan_autotune(cashash_ctx* c, cashash_plan* pl, const double* F_dev,
   const int prof = c->profiling;
   c->profiling = 0;
   std::vector<cashash_tuning> cand;
-  for (uint32_t ctas : {0u, 1u})
-    for (uint32_t tile : {4u, 2u}) {
-      cashash_tuning t{};
-      t.kernel = CASHASH_KERNEL_JOIN;
-      t.tile = tile;
-      t.ctas_per_sm = ctas;
-      cand.push_back(t);
-    }
+  for (uint32_t ctas : {0u, 1u}) {
+    cashash_tuning t{};
+    t.kernel = CASHASH_KERNEL_JOIN;
+    t.tile = 4;
+    t.ctas_per_sm = ctas;
+    cand.push_back(t);
+  }
   for (uint32_t ctas : {0u, 1u}) {
     cashash_tuning t{};
     t.kernel = CASHASH_KERNEL_JOIN_TC;

@@ -290,12 +290,14 @@ struct MatchArgs {
 // Bucket-join matching (batched schedule): calibration of missing per-pair
 // thresholds (launch_join_calibrate), then the join kernel over items = pairs.
 cudaError_t launch_join_calibrate(const MatchArgs& a, cudaStream_t s);
-// ntc: candidate tiles of 8 columns held in registers (2 or 4).
-cudaError_t launch_join(const MatchArgs& a, uint32_t grid, uint32_t ntc, cudaStream_t s);
+cudaError_t launch_join(const MatchArgs& a, uint32_t grid, cudaStream_t s);
 // Resident CTAs of the join for n_items pairs (at most ctas_per_sm per SM when
 // non-zero); 0 when the join does not apply (the largest query image exceeds
-// its shared memory).  The band form runs with 4 candidate tiles.
-uint32_t join_grid(const KParams& kp, uint32_t na_max, uint32_t n_items, uint32_t ntc, uint32_t ctas_per_sm);
+// its shared memory).
+uint32_t join_grid(const KParams& kp, uint32_t na_max, uint32_t n_items, uint32_t ctas_per_sm);
+// The band form of both (epi_px >= 0).
+uint32_t join_band_grid(const KParams& kp, uint32_t na_max, uint32_t n_items, uint32_t ctas_per_sm);
+cudaError_t launch_join_band(const MatchArgs& a, uint32_t grid, cudaStream_t s);
 // The bucket join on tcgen05 tensor cores (same results as launch_join):
 // resident CTAs for n_items pairs (at most 2 per SM, ctas_per_sm when
 // non-zero and smaller), 0 when the largest query image exceeds its shared

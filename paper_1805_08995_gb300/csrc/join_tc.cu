@@ -46,7 +46,7 @@ constexpr uint32_t TJ_SCRATCH_WORDS = 16;     // epilogue: one 16-column chunk p
 // and distances][column indices][row query, run begin, run end][bucket
 // offsets of A and B][survivor counters].
 __host__ __device__ inline size_t tj_op_bytes(int KC) {
-  const size_t ops = TJ_A_BYTES + TJ_B_BYTES, fin = (size_t)2 * KC * JT * 4;
+  const size_t ops = TJ_A_BYTES + TJ_B_BYTES, fin = (size_t)2 * join_kp(KC) * JT * 4;
   return ops > fin ? ops : fin;
 }
 __host__ __device__ inline size_t tj_smem_bytes(int KC, uint32_t na_max) {
@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(JT, 2) k_join_tc(MatchArgs a) {
   uint32_t* s_boff = s_aoff + 260;                            // [260] bucket offsets of B, table t
   uint32_t* cnt_s = s_boff + 260;                             // [na_max] survivor counters
   uint32_t* key_s = reinterpret_cast<uint32_t*>(tsm);         // finalisation (aliases the operands)
-  uint32_t* dist_s = key_s + KC * JT;
+  uint32_t* dist_s = key_s + join_kp(KC) * JT;
   uint32_t* seg = a.jqueue + (size_t)blockIdx.x * a.na_max * JSEG;
   const uint32_t h_user = TAU ? kp.tau : 128u;
   float4* lines = EPI ? a.jline + (size_t)blockIdx.x * a.na_max : nullptr;
