@@ -55,7 +55,7 @@ __host__ __device__ inline uint64_t join_block(uint64_t n) {
   return 1040u + 4u * ((n + 3) / 4 * 4) + 16u * n;
 }
 
-// Bucket join with the band: per CTA, FP32 (a, b, c, w_lo) of each query's line, then w_hi.
+// Bucket join with the band: per pair in flight, FP32 (a, b, c, w_lo) of each query's line, then w_hi.
 __host__ __device__ inline uint64_t jline_stride(uint64_t na_max) { return na_max + (na_max + 3) / 4; }
 
 // Per-row constants of the projection (Sec. 5.1) derived from R and the centre.
@@ -185,25 +185,32 @@ __device__ __forceinline__ int epi_test32(float a, float b, float c, float r, fl
   return 2;
 }
 
-// Thresholds on |n|, n = fl32(a x' + b y' + c) as two FMAs (a, b, c the FP32 roundings of the
-// FP64 line), that decide epi_keep for every candidate of an image whose key-points satisfy
-// |x'| <= mx and |y'| <= my: |n| <= w_lo keeps, |n| >= w_hi drops, anything between (or NaN) is
-// left to the FP64 expression.  With u = 2^-24 and S = |a| mx + |b| my + |c|, the two FMA
-// roundings and the roundings of a, b, c give |n - num| <= 3 u S (1 + u) + 3 * 2^-53 S, num the
-// FP64 numerator; the FP64 square num^2 <= rhs holds whenever |num| <= sqrt(rhs) (1 - 2^-40) and
-// fails whenever |num| >= sqrt(rhs) (1 + 2^-40), since the roundings of the square, of the root
-// and of these bounds are all below 2^-50 relative.  The absolute 1e-30 covers FP32 underflow;
-// lines that are not finite, or so large that n could overflow, leave every candidate to FP64.
-__device__ __forceinline__ void band_thresholds(const EpiQ& e, float mx, float my, float& wlo, float& whi) {
-  wlo = -INFINITY;
-  whi = INFINITY;
-  const double t = sqrt(e.rhs);
-  const double S = fabs((double)e.a) * (double)mx + fabs((double)e.b) * (double)my + fabs((double)e.c);
-  const double en = 3.02 * 0x1p-24 * S + 1e-30;
-  const double lo = t * (1.0 - 0x1p-40) - en, hi = t * (1.0 + 0x1p-40) + en;
-  if (S < 1e30 && isfinite(lo) && isfinite(hi)) {
-    wlo = __double2float_rd(lo);
-    whi = __double2float_ru(hi);
+// The band test of one query for every candidate of an image whose key-points satisfy |x'| <= mx and
+// |y'| <= my: the FP32 roundings a, b, c of the FP64 line and two thresholds on |n|, n = fl32(a x' + b y' + c)
+// as two FMAs: |n| <= lo keeps, |n| >= hi drops, anything between (or NaN) is left to the FP64 expression.
+// With u = 2^-24 and S = |a| mx + |b| my + |c|, the two FMA roundings and the roundings of a, b, c give
+// |n - num| <= 3 u S (1 + u) + 3 * 2^-53 S, num the FP64 numerator; the FP64 square num^2 <= rhs holds whenever
+// |num| <= sqrt(rhs) (1 - 2^-40) and fails whenever |num| >= sqrt(rhs) (1 + 2^-40), since the roundings of the
+// square and of the root are below 2^-50 relative.  The thresholds are FP32 with every step rounded outwards
+// (FP64 only where the line itself needs it: the FP64 pipe is narrow); sqrt(rhs) carries a relative margin of
+// 2^-22, S a factor 1.81e-7 > 3.02 u, and the absolute 1e-30 covers FP32 underflow: a and b that round to zero or
+// to subnormal numbers are off by at most 2^-150, times |x'| < 1e14.  Lines that are not finite, or so large that n
+// could overflow, and larger key-points leave every candidate to FP64.
+__device__ __forceinline__ void band_line(const double* F, float2 pq, double dd, float mx, float my, float4& l,
+                                          float& hi) {
+  double la, lb, lc, rhs;
+  epi_line(F, pq, dd, la, lb, lc, rhs);
+  l.x = __double2float_rn(la);
+  l.y = __double2float_rn(lb);
+  l.z = __double2float_rn(lc);
+  const float t0 = __fsqrt_rd(__double2float_rd(rhs)), t1 = __fsqrt_ru(__double2float_ru(rhs));
+  const float S = __fmaf_ru(fabsf(l.x), mx, __fmaf_ru(fabsf(l.y), my, fabsf(l.z)));
+  const float en = __fmaf_ru(1.81e-7f, S, 1e-30f);
+  l.w = __fsub_rd(__fmul_rd(t0, 1.0f - 0x1p-22f), en);
+  hi = __fadd_ru(__fmul_ru(t1, 1.0f + 0x1p-22f), en);
+  if (!(S < 1e30f) || !(t1 < 1e30f) || !(fmaxf(mx, my) < 1e14f)) {
+    l.w = -INFINITY;
+    hi = __int_as_float(0x7FFFFFFF);  // NaN: no |n|, infinite ones included, reaches it
   }
 }
 
@@ -283,7 +290,7 @@ struct MatchArgs {
   const uint8_t* join;       // bucket join: table buffer holding the bucket-sorted tables
   uint32_t* jqueue;          // bucket join: [grid][na_max][JSEG] survivor lists
   uint32_t* jhist;           // bucket join: [P][HBINS] k-th Hamming distances seen per pair
-  float4* jline;             // bucket join with the band: per CTA jline_stride(na_max) float4s of query lines
+  float4* jline;             // bucket join with the band: per pair in flight jline_stride(na_max) float4s of query lines
   uint32_t na_max;           // bucket join: largest query image of the plan
   KParams kp;
 };
@@ -295,9 +302,6 @@ cudaError_t launch_join(const MatchArgs& a, uint32_t grid, cudaStream_t s);
 // non-zero); 0 when the join does not apply (the largest query image exceeds
 // its shared memory).
 uint32_t join_grid(const KParams& kp, uint32_t na_max, uint32_t n_items, uint32_t ctas_per_sm);
-// The band form of both (epi_px >= 0).
-uint32_t join_band_grid(const KParams& kp, uint32_t na_max, uint32_t n_items, uint32_t ctas_per_sm);
-cudaError_t launch_join_band(const MatchArgs& a, uint32_t grid, cudaStream_t s);
 // The bucket join on tcgen05 tensor cores (same results as launch_join):
 // resident CTAs for n_items pairs (at most 2 per SM, ctas_per_sm when
 // non-zero and smaller), 0 when the largest query image exceeds its shared

@@ -1,6 +1,5 @@
 // Batched matching as a bucket join: Steps 1-4 of Sec. 3.1 (+ the Sec. 6
-// threshold tau) organised around the lookup tables.  (With the Sec. 7.2 band:
-// join_band.cu.)
+// threshold tau, + the Sec. 7.2 band) organised around the lookup tables.
 //
 // Step 1 pairs a query with exactly the candidates that share its bucket in
 // some table, so for table t and short code v the work is the dense block
@@ -18,6 +17,10 @@
 // query whose list overflowed, or that holds fewer than k distinct survivors
 // while the guess turned some candidate away, is left PENDING for the exact
 // fallback kernel, so results never depend on the guess.
+//
+// With the band (EPI) a candidate outside it is no candidate at all, so there is
+// no Hamming guess, and the band test, cheaper than a Hamming distance and passed
+// by few, comes first.
 //
 // Why the distances are population counts and not a tensor-core contraction: on
 // sm_103a an FP8 mma.sync executes as two tensor instructions after converting
@@ -50,10 +53,15 @@ constexpr uint32_t CAL_MARGIN = 1; // calibration: Hamming margin over the secon
 constexpr int JNT = 512;       // threads of a CTA (two per SM; 4 x 256: 17.3 ms, 1 x 1024: 16.9 against 16.7)
 constexpr uint32_t JCOL = 64;  // candidates of a bucket staged in shared memory at a time, per warp
 
-// Shared memory of a warp: the staged candidates' codes and indices.
+// Shared memory of a warp: the staged candidates' codes and indices, and with the band their key-points.
+template <bool EPI>
 struct JoinWarp {
   uint4 col[JCOL];
   uint32_t colj[JCOL];
+};
+template <>
+struct JoinWarp<true> : JoinWarp<false> {
+  float2 colp[JCOL];
 };
 
 // The 2^lg CTAs of a cluster share a pair: 32 queries at a time, tile q / 32 belongs to CTA (q / 32) % 2^lg,
@@ -63,8 +71,9 @@ __host__ __device__ inline uint32_t join_own(uint32_t na, uint32_t lg) {
 }
 // Shared memory of a CTA: its counters, then the warps' parts and the bucket offsets ([2][T][2^m + 1]), or the
 // finalisation's keys and distances.
-__host__ __device__ inline size_t join_smem_bytes(int KC, uint32_t T, uint32_t na_max, uint32_t lg) {
-  const size_t fin = (size_t)2 * join_kp(KC) * JNT * 4, scan = (JNT / 32) * sizeof(JoinWarp) + (size_t)2 * T * 257 * 4;
+__host__ __device__ inline size_t join_smem_bytes(int KC, uint32_t T, uint32_t na_max, uint32_t lg, bool epi) {
+  const size_t fin = (size_t)2 * join_kp(KC) * JNT * 4,
+               scan = (JNT / 32) * (epi ? sizeof(JoinWarp<true>) : sizeof(JoinWarp<false>)) + (size_t)2 * T * 257 * 4;
   return join_own(na_max, lg) + (fin > scan ? fin : scan);
 }
 
@@ -116,7 +125,7 @@ __device__ __forceinline__ void scan4(uint4 q, uint32_t& off, int h_thr, const u
 
 // The queries qs .. qs + nq of A's bucket against the nb staged candidates.
 template <bool CL>
-__device__ __forceinline__ void scan_rows(const JoinWarp& w, const JView& A, uint32_t qs, uint32_t nq, uint32_t nb,
+__device__ __forceinline__ void scan_rows(const JoinWarp<false>& w, const JView& A, uint32_t qs, uint32_t nq, uint32_t nb,
                                           uint32_t h_thr, const JoinLists<CL>& L, int lane) {
   for (; nq > 16; qs += min(nq, 32u), nq -= min(nq, 32u)) {
     if ((uint32_t)lane < nq) {
@@ -167,7 +176,67 @@ __device__ __forceinline__ void scan_rows(const JoinWarp& w, const JView& A, uin
   }
 }
 
-template <int KC, bool CL>
+// The same inside the band of Sec. 7.2: a candidate counts when its distance from the query's epipolar line is
+// inside the band and H <= h_thr (tau).  Few candidates do, so 32 at a time take two FMAs and a compare with the
+// line's upper threshold (band_line), and the lane's bits that are left take the rest: the lower threshold,
+// the FP64 expression in between, the Hamming distance and the store.
+// The distance comes last since the band turns nearly all away; with FP8 mma.sync blocks, whose distances come for
+// all, and the band test on every slot of the padded blocks, it took 2.72 warp instructions per entry against 0.90.
+// 300 pairs of views with about 8,000 key-points: 2.43 -> 0.79 ms; all overlapping pairs of 160 such views:
+// 26.9 -> 9.0 ms.  Bound by issue (54 % of the slots, 23 of 32 threads in an instruction) and latency.
+struct BandRows {
+  const float4* line;  // per query: FP32 a, b, c and the lower threshold on |a x' + b y' + c|
+  const float* hi;     // ... and the upper one
+  const double* F;
+  const float2* kpa;   // key-points of the query image
+  double dd;
+};
+template <bool CL>
+__device__ __forceinline__ void scan_rows_band(const JoinWarp<true>& w, const JView& A, uint32_t qs, uint32_t nq,
+                                               uint32_t nb, uint32_t h_thr, const JoinLists<CL>& L, const BandRows& R,
+                                               int lane) {
+  for (uint32_t r0 = 0; r0 < nq; r0 += 32) {
+    if (r0 + lane < nq) {
+      const uint4 code = __ldg(A.rec + qs + r0 + lane);
+      const uint32_t q = __ldg(A.idx + qs + r0 + lane);
+      const float4 l = __ldcg(R.line + q);
+      const float hi = __ldcg(R.hi + q);
+      uint32_t* list = L.seg + (size_t)q * JSEG;
+      uint8_t* cnt = L.count(q);
+      uint32_t n = *cnt;
+#pragma unroll 1
+      for (uint32_t c0 = 0; c0 < nb; c0 += 32) {
+        uint32_t m = 0;
+#pragma unroll
+        for (uint32_t u = 0; u < 32; u += 8) {
+          if (c0 + u >= nb) break;  // (the last eight may read past nb: masked below)
+#pragma unroll
+          for (uint32_t e = 0; e < 8; ++e) {
+            const float2 p = w.colp[c0 + u + e];
+            const float d = fabsf(fmaf(l.x, p.x, fmaf(l.y, p.y, l.z)));
+            if (!(d >= hi)) m |= 1u << (u + e);
+          }
+        }
+        if (nb - c0 < 32) m &= (1u << (nb - c0)) - 1u;
+        while (m) {
+          const uint32_t c = c0 + __ffs(m) - 1;
+          m &= m - 1;
+          const float2 p = w.colp[c];
+          const uint32_t h = jt_hamming(w.col[c], code);
+          if (h > h_thr) continue;
+          if (!(fabsf(fmaf(l.x, p.x, fmaf(l.y, p.y, l.z))) <= l.w) && !epi_keep_fp64_F(R.F, __ldg(R.kpa + q), R.dd, p))
+            continue;
+          if (n < JSEG) list[n] = (h << 24) + w.colj[c];
+          ++n;
+        }
+      }
+      *cnt = (uint8_t)min(n, JSEG + 1u);
+    }
+    __syncwarp();
+  }
+}
+
+template <int KC, bool CL, bool EPI>
 __global__ void __launch_bounds__(JNT, 2) k_join(MatchArgs a) {
   extern __shared__ __align__(16) uint8_t jsm[];
   __shared__ uint32_t s_item, s_tau, s_task[CASHASH_MAX_TABLES];
@@ -185,14 +254,18 @@ __global__ void __launch_bounds__(JNT, 2) k_join(MatchArgs a) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   uint8_t* cnt_s = jsm;
   uint8_t* work = jsm + join_own(a.na_max, lg);
-  JoinWarp& w = reinterpret_cast<JoinWarp*>(work)[warp];
-  uint32_t* off_s = reinterpret_cast<uint32_t*>(reinterpret_cast<JoinWarp*>(work) + JNT / 32);
+  JoinWarp<EPI>& w = reinterpret_cast<JoinWarp<EPI>*>(work)[warp];
+  uint32_t* off_s = reinterpret_cast<uint32_t*>(reinterpret_cast<JoinWarp<EPI>*>(work) + JNT / 32);
   uint32_t* key_s = reinterpret_cast<uint32_t*>(work);
   uint32_t* dist_s = key_s + join_kp(KC) * JNT;
   const JoinLists<CL> L{a.jqueue + (size_t)(blockIdx.x >> lg) * a.na_max * JSEG, cnt_s, lg};
   const uint32_t* item0 = CL ? cl.map_shared_rank(&s_item, 0) : &s_item;
   uint32_t* task0 = CL ? cl.map_shared_rank(s_task, 0) : s_task;
   const uint32_t h_user = kp.tau < kp.code_bits ? kp.tau : 128u;  // Sec. 6: keys with H > tau are no candidates
+  __shared__ uint32_t s_kx, s_ky;  // band: the largest |x'|, |y'| of the candidate image
+  float4* lines = EPI ? a.jline + (size_t)(blockIdx.x >> lg) * jline_stride(a.na_max) : nullptr;
+  float* lhi = EPI ? reinterpret_cast<float*>(lines + a.na_max) : nullptr;
+  const double dd = kp.epi_px * kp.epi_px;
   const uint32_t nbo = T * (nbk + 1), nsp = kp.bits_per_table < 6 ? 6 - kp.bits_per_table : 0;
 
   for (;;) {
@@ -208,9 +281,12 @@ __global__ void __launch_bounds__(JNT, 2) k_join(MatchArgs a) {
     sync();
     const uint32_t it = *item0;  // pair index
     if (it == 0xFFFFFFFFu) break;
-    if (tid == 0) s_P = a.pairs[it];
+    if (tid == 0) {
+      s_P = a.pairs[it];
+      s_kx = s_ky = 0u;
+    }
     __syncthreads();
-    if (warp == 0) {
+    if (!EPI && warp == 0) {
       const uint32_t gs = pair_threshold(a, it, lane);
       if (lane == 0) s_tau = gs;
     }
@@ -223,11 +299,40 @@ __global__ void __launch_bounds__(JNT, 2) k_join(MatchArgs a) {
       off_s[i] = __ldg(jview(a.join, s_P.ajoin, s_P.nA, t).off + v);
       off_s[nbo + i] = __ldg(jview(a.join, s_P.bjoin, s_P.nB, t).off + v);
     }
+    if constexpr (EPI) {  // (non-negative floats order as integers)
+      const float2* kpb = reinterpret_cast<const float2*>(a.kpts) + s_P.b0;
+      float mx = 0.f, my = 0.f;
+      for (uint32_t j = tid; j < s_P.nB; j += JNT) {
+        const float2 pc = __ldg(kpb + j);
+        mx = fmaxf(mx, fabsf(pc.x));
+        my = fmaxf(my, fabsf(pc.y));
+      }
+      mx = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, __float_as_uint(mx)));
+      my = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, __float_as_uint(my)));
+      if (lane == 0) {
+        atomicMax(&s_kx, __float_as_uint(mx));
+        atomicMax(&s_ky, __float_as_uint(my));
+      }
+    }
     __syncthreads();
     uint32_t h_thr = h_user;
-    const uint32_t ts = s_tau;  // 0: no guess; else threshold + 1
-    if (ts != 0 && ts - 1u < h_thr) h_thr = ts - 1u;
+    if (!EPI) {
+      const uint32_t ts = s_tau;  // 0: no guess; else threshold + 1
+      if (ts != 0 && ts - 1u < h_thr) h_thr = ts - 1u;
+    }
     const bool cut = h_thr < h_user;  // the guess may turn candidates away
+    const float2* kpa = EPI ? reinterpret_cast<const float2*>(a.kpts) + s_P.a0 : nullptr;
+    const BandRows band{lines, lhi, EPI ? a.F + 9 * (size_t)it : nullptr, kpa, dd};
+    if constexpr (EPI) {  // the queries' lines, spread over the cluster
+      for (uint32_t q = rank * JNT + tid; q < s_P.nA; q += JNT << lg) {
+        float4 l;
+        float hi;
+        band_line(band.F, __ldg(kpa + q), dd, __uint_as_float(s_kx), __uint_as_float(s_ky), l, hi);
+        lines[q] = l;
+        lhi[q] = hi;
+      }
+      sync();
+    }
 
     // ---- scan: a table at a time (a query lies in one bucket of it, so its list and counter have one
     // writer), one warp per bucket (or part of its queries, when there are few buckets), one query per lane
@@ -253,10 +358,13 @@ __global__ void __launch_bounds__(JNT, 2) k_join(MatchArgs a) {
           for (uint32_t u = 0; u < JCOL; u += 32)
             if (u + lane < nb) {
               w.col[u + lane] = __ldg(s_B[t].rec + cs + c0 + u + lane);
-              w.colj[u + lane] = __ldg(s_B[t].idx + cs + c0 + u + lane);
+              const uint32_t jj = __ldg(s_B[t].idx + cs + c0 + u + lane);
+              w.colj[u + lane] = jj;
+              if constexpr (EPI) w.colp[u + lane] = __ldg(reinterpret_cast<const float2*>(a.kpts) + s_P.b0 + jj);
             }
           __syncwarp();
-          scan_rows(w, s_A[t], qs, nq, nb, h_thr, L, lane);
+          if constexpr (EPI) scan_rows_band(w, s_A[t], qs, nq, nb, h_thr, L, band, lane);
+          else scan_rows(w, s_A[t], qs, nq, nb, h_thr, L, lane);
         }
       }
       sync();
@@ -265,12 +373,12 @@ __global__ void __launch_bounds__(JNT, 2) k_join(MatchArgs a) {
     // ---- finalise: top-k of the survivors, distances, ratio test ----
     for (uint32_t k = warp; ((k << lg) + rank) * 32 < s_P.nA; k += JNT / 32) {
       const uint32_t q = ((k << lg) + rank) * 32 + lane;
-      finalise_warp<KC, false>(a, s_P, it, cut, q, q < s_P.nA, q < s_P.nA ? cnt_s[k * 32 + lane] : 0u,
+      finalise_warp<KC, EPI>(a, s_P, it, cut, q, q < s_P.nA, q < s_P.nA ? cnt_s[k * 32 + lane] : 0u,
                                L.seg + (size_t)q * JSEG, key_s + warp * 32 * join_kp(KC),
                                dist_s + warp * 32 * join_kp(KC), s_hist);
     }
     __syncthreads();
-    if (!a.tau_fixed)
+    if (!EPI && !a.tau_fixed)
       for (uint32_t b = tid; b < HBINS; b += JNT)
         if (s_hist[b]) atomicAdd(a.jhist + (size_t)it * HBINS + b, s_hist[b]);
   }
@@ -345,17 +453,19 @@ __global__ void __launch_bounds__(CAL_SAMPLES) k_join_calibrate(MatchArgs a) {
 // ---------------------------------------------------------------------------
 namespace {
 
-// The function pointer of the instantiation for k (k_join, or k_join_calibrate).
 using JoinKernel = void (*)(MatchArgs);
-template <bool CL>
+template <bool CL, bool EPI>
 JoinKernel join_kernel_kc(uint32_t k) {
-  return k <= 4    ? k_join<4, CL>
-         : k <= 8  ? k_join<8, CL>
-         : k <= 10 ? k_join<10, CL>
-         : k <= 16 ? k_join<16, CL>
-                   : k_join<32, CL>;
+  return k <= 4    ? k_join<4, CL, EPI>
+         : k <= 8  ? k_join<8, CL, EPI>
+         : k <= 10 ? k_join<10, CL, EPI>
+         : k <= 16 ? k_join<16, CL, EPI>
+                   : k_join<32, CL, EPI>;
 }
-JoinKernel join_kernel(uint32_t k, uint32_t lg) { return lg ? join_kernel_kc<true>(k) : join_kernel_kc<false>(k); }
+JoinKernel join_kernel(uint32_t k, uint32_t lg, bool epi) {
+  if (epi) return lg ? join_kernel_kc<true, true>(k) : join_kernel_kc<false, true>(k);
+  return lg ? join_kernel_kc<true, false>(k) : join_kernel_kc<false, false>(k);
+}
 JoinKernel calibrate_kernel(uint32_t k) {
   return k <= 4    ? k_join_calibrate<4>
          : k <= 8  ? k_join_calibrate<8>
@@ -391,15 +501,15 @@ uint32_t join_lg(uint32_t n_items, int nsm) {
 }  // namespace
 
 uint32_t join_grid(const KParams& kp, uint32_t na_max, uint32_t n_items, uint32_t ctas_per_sm) {
-  if (kp.epi_px >= 0.0) return join_band_grid(kp, na_max, n_items, ctas_per_sm);
+  const bool epi = kp.epi_px >= 0.0;
   // query images whose 32-bit counters and keys would exceed a CTA's shared memory take the per-query kernel
   if ((size_t)4 * ((na_max + 3) / 4 * 4) + (size_t)2 * join_kc(kp.top_k) * JT * 4 + 4096 > 227u * 1024u) return 0;
   int dev = 0, nsm = 0, ncl = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const uint32_t lg = join_lg(n_items, nsm);
-  const size_t smem = join_smem_bytes(join_kc(kp.top_k), kp.n_tables, na_max, lg);
-  const JoinKernel kern = join_kernel(kp.top_k, lg);
+  const size_t smem = join_smem_bytes(join_kc(kp.top_k), kp.n_tables, na_max, lg, epi);
+  const JoinKernel kern = join_kernel(kp.top_k, lg, epi);
   const uint32_t ctas = join_resident(kern, smem, lg ? 1u : n_items, ctas_per_sm, JNT);
   if (!lg || !ctas) return ctas;
   cudaLaunchConfig_t cfg{};
@@ -425,20 +535,20 @@ cudaError_t launch_join_calibrate(const MatchArgs& a, cudaStream_t s) {
 
 cudaError_t launch_join(const MatchArgs& a, uint32_t grid, cudaStream_t s) {
   if (a.n_items == 0 || grid == 0) return cudaSuccess;
-  if (a.kp.epi_px >= 0.0) return launch_join_band(a, grid, s);
+  const bool epi = a.kp.epi_px >= 0.0;
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const uint32_t lg = join_lg(a.n_items, nsm);
-  const size_t smem = join_smem_bytes(join_kc(a.kp.top_k), a.kp.n_tables, a.na_max, lg);
+  const size_t smem = join_smem_bytes(join_kc(a.kp.top_k), a.kp.n_tables, a.na_max, lg, epi);
   if (!lg) {
-    join_kernel(a.kp.top_k, 0)<<<grid, JNT, smem, s>>>(a);
+    join_kernel(a.kp.top_k, 0, epi)<<<grid, JNT, smem, s>>>(a);
     return cudaGetLastError();
   }
   cudaLaunchConfig_t cfg{};
   cudaLaunchAttribute at{};
   join_config(cfg, at, grid << lg, lg, smem, s);
-  return cudaLaunchKernelEx(&cfg, join_kernel(a.kp.top_k, lg), a);
+  return cudaLaunchKernelEx(&cfg, join_kernel(a.kp.top_k, lg, epi), a);
 }
 
 }  // namespace chx

@@ -1,7 +1,7 @@
-// Helpers shared by the bucket-join kernels (join.cu, the band form in
-// join_band.cu, the tcgen05 form in join_tc.cu): the top-k insertion network, the
-// view of one image's bucket-sorted table, the per-pair Hamming threshold, the
-// finalisation of a pair's survivor lists, and the launch sizes.
+// Helpers shared by the two bucket-join kernels (join.cu, and the tcgen05 form in
+// join_tc.cu): the top-k insertion network, the view of one image's bucket-sorted
+// table, the per-pair Hamming threshold, the finalisation of a pair's survivor
+// lists, and the launch sizes.
 #pragma once
 
 #include <cuda_fp16.h>
@@ -10,7 +10,7 @@
 
 namespace chx {
 
-constexpr int JT = 256;  // threads of a CTA of the band and tcgen05 forms
+constexpr int JT = 256;  // threads of a CTA of the tcgen05 form
 
 template <int KC>
 __device__ __forceinline__ void jt_insert(uint32_t (&top)[KC], uint32_t k) {
@@ -259,22 +259,6 @@ __device__ __forceinline__ void join_finalise(const MatchArgs& a, const PairInfo
     const uint32_t q = q0 + threadIdx.x;
     finalise_warp<KC, EPI>(a, P, it, cut, q, q < P.nA, q < P.nA ? cnt_s[q] : 0u, seg + (size_t)q * JSEG, key_s + w,
                            dist_s + w, s_hist);
-  }
-}
-
-// Bucket offsets of join task `task` (table task / nbk, bucket task % nbk) in
-// both images; zeros past the last task.
-__device__ __forceinline__ void load_offsets(const uint8_t* join, const PairInfo& P, uint64_t ablk, uint64_t bblk,
-                                             uint32_t nbk, uint32_t ntask, uint32_t task, uint32_t (&o)[4]) {
-  o[0] = o[1] = o[2] = o[3] = 0u;
-  if (task < ntask) {
-    const uint32_t t = task / nbk, v = task - t * nbk;
-    const uint32_t* ao = reinterpret_cast<const uint32_t*>(join + P.ajoin + t * ablk) + v;
-    const uint32_t* bo = reinterpret_cast<const uint32_t*>(join + P.bjoin + t * bblk) + v;
-    o[0] = __ldg(ao);
-    o[1] = __ldg(ao + 1);
-    o[2] = __ldg(bo);
-    o[3] = __ldg(bo + 1);
   }
 }
 
