@@ -944,8 +944,15 @@ int enqueue_match(cashash_ctx* c, cashash_plan* pl, const double* F_dev, uint64_
     }
   } else {
     StageTimer tm(c, CASHASH_STAGE_MATCH, stream, capturing);
+    bool after = false;
     for (uint32_t i = 0; i < P; ++i) {
       if (!pl->count[i]) continue;
+      if (match_pair_by_warps(c->kp, pl->info[i].nA, pl->info[i].nB)) {
+        CK(launch_match_pair(a, i, pl->info[i], after, stream));
+        after = true;
+        continue;
+      }
+      after = false;
       a.items = pl->d_items + pl->first[i];
       a.n_items = pl->count[i];
       a.item_ctr = pl->d_item_ctr + i;

@@ -11,7 +11,7 @@
 // set), and ordered by (Hamming, index).
 //
 // Two forms of the selection:
-//  * direct (one pair per launch): every key below the current k-th key goes
+//  * direct (one pair per launch, the largest pairs only: match_pair_by_warps below): every key below the current k-th key goes
 //    through a branch-free insertion network in registers that also drops a
 //    key equal to one already kept;
 //  * speculative (batched): the hot loop only appends keys below a threshold
@@ -272,25 +272,146 @@ __global__ void __launch_bounds__(TPB, (TPB <= 512 ? 2 : 1)) k_match(MatchArgs a
 }
 
 // ---------------------------------------------------------------------------
-// Exact fallback for PENDING queries, one warp per query.  Warps stream the
-// per-query result array (128 entries per step, coalesced); for each PENDING
-// entry the warp finds its pair with a 32-way search over the pairs' first
-// result index, then walks the query's buckets in the chunked lookup tables
-// with the lanes side by side.  Each lane keeps the k smallest distinct keys
-// it met; the warp merges them by k rounds of minimum extraction (equal keys
-// of several lanes leave together, so a point met through several tables
-// counts once), k lanes compute the exact distances and lane 0 applies the
-// ratio test.
+// Exact matching, one warp per query: PENDING queries of the batched kernels (k_match_fallback; all queries of a plan
+// in the warp-per-query configuration) and the queries of one pair (k_match_pair, the per-pair schedule).
+//
+// One query: the candidates of a bucket lie next to each other in the image's bucket-sorted tables, codes inline.
+// The lanes fetch the T offset pairs at once, number the candidates through all tables and take 4 x 32 at a time
+// side by side, so a query costs a handful of dependent memory latencies whatever T is (the chunked tables have a
+// list per chunk and table, each two latencies before the code itself).  Each lane keeps the k smallest distinct
+// keys it met; the warp merges them by k rounds of minimum extraction (equal keys of several lanes leave together,
+// so a point met through several tables counts once); 8 lanes take each ranked candidate's row.  Small pairs are
+// bound by the latencies, large ones by issue and L2 (20 B per candidate, about 3 ps at 20,000 queries with long
+// buckets).  A pass over one pair with CASHASH_KERNEL_WARP, chunked tables -> now: 2,000 x 2,000 features 18.6 ->
+// 14.6 us, 8,000 45 -> 34.6, 20,000 166 -> 93; the fallback of 4,950 pairs of 8k x 8k 0.62 -> 0.42 ms.
 // ---------------------------------------------------------------------------
-// One query g of the per-query result array, by one warp (exact): the pair
-// holding g, the query's buckets walked with the lanes side by side, the
-// merge of the lanes' k smallest distinct keys, distances and the ratio test.
+template <int KC, bool EPI>
+__device__ __forceinline__ void warp_query(const MatchArgs& a, uint32_t pair, const PairInfo& P, uint32_t q, int lane,
+                                           uint32_t thr_user, double dd) {
+  constexpr uint32_t FULL = 0xFFFFFFFFu;
+  const KParams& kp = a.kp;
+  const uint32_t T = kp.n_tables, K = kp.top_k;
+  const uint64_t fa = P.a0 + q;
+  const int grp = lane >> 3, sub = lane & 7;
+  const uint4 qc = __ldg(reinterpret_cast<const uint4*>(a.codes) + fa);
+  const uint4 av = __ldg(reinterpret_cast<const uint4*>(a.desc + fa * DIM) + sub);
+  const uint64_t blk = join_block(P.nB);
+  const uint8_t* jt = a.tables + P.bjoin;
+  uint32_t s0 = 0, n = 0;  // lane t: the first entry and the number of entries of the query's bucket in table t
+  if ((uint32_t)lane < T) {
+    const uint32_t* off = reinterpret_cast<const uint32_t*>(jt + (uint64_t)lane * blk) + __ldg(a.buckets + fa * 8 + lane);
+    s0 = __ldg(off);
+    n = __ldg(off + 1) - s0;
+  }
+  uint32_t end = n;  // inclusive prefix over the tables
+#pragma unroll
+  for (int o = 1; o < CASHASH_MAX_TABLES; o <<= 1) {
+    const uint32_t v = __shfl_up_sync(FULL, end, o);
+    if (lane >= o) end += v;
+  }
+  const uint32_t adj = s0 - (end - n);  // entry of table t = number + adj
+  uint32_t e[CASHASH_MAX_TABLES];
+#pragma unroll
+  for (int t = 0; t < CASHASH_MAX_TABLES; ++t) e[t] = __shfl_sync(FULL, end, t);
+  const uint32_t total = e[CASHASH_MAX_TABLES - 1];
+  EpiQ eq{};
+  if (EPI) eq = epi_query(a.F + 9 * (size_t)pair, __ldg(reinterpret_cast<const float2*>(a.kpts) + fa), dd);
+  const float2* kb = reinterpret_cast<const float2*>(a.kpts) + P.b0;
+  const uint64_t rec0 = 1040 + 4 * (uint64_t)((P.nB + 3) / 4 * 4);
+  uint32_t top[KC];
+#pragma unroll
+  for (int s = 0; s < KC; ++s) top[s] = KEY_INF;
+  constexpr int U = 4;
+  for (uint32_t p0 = 0; p0 < total; p0 += 32 * U) {
+    uint4 c[U];
+    uint32_t j[U];
+    float2 pc[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      j[u] = 0xFFFFFFFFu;
+      if (p0 + 32 * u >= total) continue;
+      const uint32_t p = p0 + 32 * u + lane;
+      int t = 0;
+#pragma unroll
+      for (int i = 0; i + 1 < CASHASH_MAX_TABLES; ++i) t += p >= e[i] ? 1 : 0;
+      const uint32_t x = p + __shfl_sync(FULL, adj, t);
+      if (p < total) {
+        const uint8_t* b = jt + (uint64_t)t * blk;
+        j[u] = __ldg(reinterpret_cast<const uint32_t*>(b + 1040) + x);
+        c[u] = __ldg(reinterpret_cast<const uint4*>(b + rec0) + x);
+      }
+    }
+    if (EPI) {
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (j[u] != 0xFFFFFFFFu) pc[u] = __ldg(kb + j[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (p0 + 32 * u >= total) break;
+      if (j[u] == 0xFFFFFFFFu) continue;
+      const uint32_t key = (hamming128(c[u], qc) << 24) | j[u];
+      if (key >= thr_user || key >= top[KC - 1]) continue;
+      if (EPI && !epi_keep_fast(eq, pc[u])) continue;
+      topk_insert<KC>(top, key);
+    }
+  }
+  // merge: round r leaves the r-th smallest distinct key in lane r
+  uint32_t mine = KEY_INF;
+  for (uint32_t r = 0; r < K; ++r) {
+    const uint32_t m = __reduce_min_sync(FULL, top[0]);
+    if (m == KEY_INF) break;  // warp-uniform
+    if ((uint32_t)lane == r) mine = m;
+    if (top[0] == m) {
+#pragma unroll
+      for (int s = 0; s + 1 < KC; ++s) top[s] = top[s + 1];
+      top[KC - 1] = KEY_INF;
+    }
+  }
+  // exact distances of the k ranked candidates (Step 4): 8 lanes per row, four rows at a time; lane r keeps row r's
+  const uint32_t nv = __popc(__ballot_sync(FULL, mine != KEY_INF));
+  const uint32_t nb2 = mine != KEY_INF ? __ldg(a.sqnorm + P.b0 + (mine & 0xFFFFFFu)) : 0u, na2 = __ldg(a.sqnorm + fa);
+  uint32_t dot = 0;
+  constexpr int ROWS = (KC + 3) / 4, RB = ROWS < 4 ? ROWS : 4;
+#pragma unroll
+  for (int i0 = 0; i0 < ROWS; i0 += RB) {
+    uint4 bv[RB];
+#pragma unroll
+    for (int i = 0; i < RB; ++i) {
+      const uint32_t key = __shfl_sync(FULL, mine, (4 * (i0 + i) + grp) & 31);
+      bv[i] = make_uint4(0u, 0u, 0u, 0u);
+      if (key != KEY_INF) bv[i] = __ldg(reinterpret_cast<const uint4*>(a.desc + (P.b0 + (key & 0xFFFFFFu)) * DIM) + sub);
+    }
+#pragma unroll
+    for (int i = 0; i < RB; ++i) {
+      uint32_t d = __dp4a(av.x, bv[i].x, 0u);
+      d = __dp4a(av.y, bv[i].y, d);
+      d = __dp4a(av.z, bv[i].z, d);
+      d = __dp4a(av.w, bv[i].w, d);
+      d += __shfl_xor_sync(FULL, d, 1);
+      d += __shfl_xor_sync(FULL, d, 2);
+      d += __shfl_xor_sync(FULL, d, 4);
+      d = __shfl_sync(FULL, d, 8 * sub & 31);  // lane r: row 4 (i0 + i) + r % 4
+      if (lane >> 2 == i0 + i) dot = d;
+    }
+  }
+  // the two smallest (distance, index), the ratio test
+  const uint32_t j = mine & 0xFFFFFFu, d = mine != KEY_INF ? na2 + nb2 - 2u * dot : 0xFFFFFFFFu;
+  const uint32_t d1 = __reduce_min_sync(FULL, d);
+  const uint32_t j1 = __reduce_min_sync(FULL, mine != KEY_INF && d == d1 ? j : 0xFFFFFFFFu);
+  const uint32_t d2 = __reduce_min_sync(FULL, d == d1 && j == j1 ? 0xFFFFFFFFu : d);
+  if (lane == 0) {
+    const bool matched = ratio_ok(kp, nv, d1, d2);
+    a.res[P.qbase + q] = matched ? j1 : NO_MATCH;
+    if (matched) atomicAdd(a.pair_cnt + pair, 1ull);
+  }
+}
+
+// The same for entry g of the per-query result array: its pair is the last with qbase <= g.
 template <int KC, bool EPI>
 __device__ __forceinline__ void fallback_query(const MatchArgs& a, uint64_t g, int lane, uint32_t thr_user,
                                                double dd) {
-  const KParams& kp = a.kp;
-  const uint32_t T = kp.n_tables, K = kp.top_k;
-  // pair: the last with qbase <= g.  32-way search; invariant: pairs[lo].qbase <= g
+  // 32-way search; invariant: pairs[lo].qbase <= g
   // and the answer lies in [lo, hi].  Lane l probes lo + 1 + l * span / 32.
   uint32_t lo = 0, hi = a.n_pairs - 1;
   while (lo < hi) {
@@ -306,80 +427,7 @@ __device__ __forceinline__ void fallback_query(const MatchArgs& a, uint64_t g, i
     }
   }
   const PairInfo P = a.pairs[lo];
-  const uint32_t q = (uint32_t)(g - P.qbase);
-  const uint4 qc = __ldg(reinterpret_cast<const uint4*>(a.codes) + P.a0 + q);
-  const uint2 qb = __ldg(reinterpret_cast<const uint2*>(a.buckets) + P.a0 + q);
-  EpiQ eq{};
-  if (EPI) eq = epi_query(a.F + 9 * (size_t)lo, __ldg(reinterpret_cast<const float2*>(a.kpts) + P.a0 + q), dd);
-  uint32_t top[KC];
-#pragma unroll
-  for (int s = 0; s < KC; ++s) top[s] = KEY_INF;
-  const uint32_t nch = (P.nB + JC - 1) / JC;
-  for (uint32_t c = 0; c < nch; ++c) {
-    const uint16_t* blk =
-        reinterpret_cast<const uint16_t*>(a.tables + (uint64_t)(P.bchunk0 + c) * chunk_bytes(T));
-    const uint4* gc = reinterpret_cast<const uint4*>(a.codes) + P.b0 + (uint64_t)c * JC;
-    for (uint32_t t = 0; t < T; ++t) {
-      const uint32_t v = (t < 4 ? (qb.x >> (8 * t)) : (qb.y >> (8 * (t - 4)))) & 0xFFu;
-      const uint32_t s0 = blk[t * OFF_STRIDE + v], s1 = blk[t * OFF_STRIDE + v + 1];
-      const uint16_t* il = blk + T * OFF_STRIDE + t * JC;
-      for (uint32_t pos = s0 + lane; pos < s1; pos += 32) {
-        const uint32_t jl = il[pos];
-        const uint32_t key = (hamming128(__ldg(gc + jl), qc) << 24) | (c * JC + jl);
-        if (key >= thr_user) continue;
-        if (EPI && !epi_keep_fast(eq, __ldg(reinterpret_cast<const float2*>(a.kpts) + P.b0 + (uint64_t)c * JC + jl)))
-          continue;
-        if (key < top[KC - 1]) topk_insert<KC>(top, key);
-      }
-    }
-  }
-  // merge: round r leaves the r-th smallest distinct key in lane r
-  uint32_t mine = KEY_INF;
-  for (uint32_t r = 0; r < K; ++r) {
-    uint32_t m = top[0];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = min(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
-    if (m == KEY_INF) break;  // warp-uniform
-    if ((uint32_t)lane == r) mine = m;
-    if (top[0] == m) {
-#pragma unroll
-      for (int s = 0; s + 1 < KC; ++s) top[s] = top[s + 1];
-      top[KC - 1] = KEY_INF;
-    }
-  }
-  // exact distances of the k ranked candidates (Step 4), ratio test
-  const uint64_t fa = P.a0 + q;
-  uint64_t dj = ~0ull;  // (d << 32) | j
-  if (mine != KEY_INF) {
-    const uint32_t j = mine & 0xFFFFFFu;
-    const uint64_t fb = P.b0 + j;
-    const uint4* arow = reinterpret_cast<const uint4*>(a.desc + fa * DIM);
-    const uint4* brow = reinterpret_cast<const uint4*>(a.desc + fb * DIM);
-    uint32_t dot = 0;
-#pragma unroll
-    for (int w = 0; w < 8; ++w) {
-      const uint4 av = __ldg(arow + w), bv = __ldg(brow + w);
-      dot = __dp4a(av.x, bv.x, dot);
-      dot = __dp4a(av.y, bv.y, dot);
-      dot = __dp4a(av.z, bv.z, dot);
-      dot = __dp4a(av.w, bv.w, dot);
-    }
-    const uint32_t d = __ldg(a.sqnorm + fa) + __ldg(a.sqnorm + fb) - 2u * dot;
-    dj = ((uint64_t)d << 32) | j;
-  }
-  const uint32_t nv = __popc(__ballot_sync(0xFFFFFFFFu, mine != KEY_INF));
-  uint64_t best = dj;  // smallest (d, j)
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) best = min(best, __shfl_xor_sync(0xFFFFFFFFu, best, o));
-  uint64_t second = dj == best ? ~0ull : dj;  // keys are distinct, so exactly one lane holds best
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) second = min(second, __shfl_xor_sync(0xFFFFFFFFu, second, o));
-  if (lane == 0) {
-    const uint32_t d1 = (uint32_t)(best >> 32), j1 = (uint32_t)best, d2 = (uint32_t)(second >> 32);
-    const bool matched = ratio_ok(kp, nv, d1, d2);
-    a.res[g] = matched ? j1 : NO_MATCH;
-    if (matched) atomicAdd(a.pair_cnt + lo, 1ull);
-  }
+  warp_query<KC, EPI>(a, lo, P, (uint32_t)(g - P.qbase), lane, thr_user, dd);
 }
 
 template <int KC, bool EPI>
@@ -397,23 +445,40 @@ __global__ void __launch_bounds__(128) k_match_fallback(MatchArgs a) {
     }
     return;
   }
-  for (uint64_t g0 = warp * 128; g0 < a.n_res; g0 += nwarp * 128) {
+  // 128 results at a time when there are many; else 32, so that a warp has at most a few pending ones in a row
+  const uint32_t nb = a.n_res > nwarp * 64 ? 4 : 1;
+  for (uint64_t g0 = warp * 32 * nb; g0 < a.n_res; g0 += nwarp * 32 * nb) {
     uint32_t pend[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (uint32_t i = 0; i < 4; ++i) {
       const uint64_t g = g0 + 32 * i + lane;
-      pend[i] = __ballot_sync(0xFFFFFFFFu, g < a.n_res && a.res[g] == PENDING);
+      pend[i] = __ballot_sync(0xFFFFFFFFu, i < nb && g < a.n_res && a.res[g] == PENDING);
     }
 #pragma unroll 1
-    for (int i = 0; i < 4; ++i) {
-      while (pend[i]) {
-        const int b = __ffs(pend[i]) - 1;
-        pend[i] &= pend[i] - 1u;
+    for (uint32_t i = 0; i < nb; ++i) {
+      uint32_t p = i == 0 ? pend[0] : i == 1 ? pend[1] : i == 2 ? pend[2] : pend[3];
+      while (p) {
+        const int b = __ffs(p) - 1;
+        p &= p - 1u;
         fallback_query<KC, EPI>(a, g0 + 32 * i + b, lane, thr_user, dd);
         __syncwarp();
       }
     }
   }
+}
+
+// One pair on its own, a warp per query: the per-pair schedule.  Launched with programmatic stream serialisation,
+// so that a pair starts when the last CTAs of the one before have started: they write disjoint results.  Every
+// thread waits for that launch at its end, so the last one completes after all of them.  120 pairs of 2,000 to 9,000
+// features: k_match (thread per query, about 40 CTAs per launch) 6.3 ms, this form 1.45 ms one launch after the
+// other, 0.84 overlapped.
+template <int KC, bool EPI>
+__global__ void __launch_bounds__(128) k_match_pair(MatchArgs a, uint32_t pair, PairInfo P) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const uint32_t thr_user = a.kp.tau < a.kp.code_bits ? ((a.kp.tau + 1u) << 24) : KEY_INF;
+  const uint32_t q = blockIdx.x * 4 + (threadIdx.x >> 5);
+  if (q < P.nA) warp_query<KC, EPI>(a, pair, P, q, threadIdx.x & 31, thr_user, a.kp.epi_px * a.kp.epi_px);
+  asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // ---------------------------------------------------------------------------
@@ -511,7 +576,7 @@ cudaError_t launch_match_fallback(const MatchArgs& a, cudaStream_t s) {
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  const uint64_t want = a.all_queries ? (a.n_res + 3) / 4 : (a.n_res + 127) / 128;  // 4 warps per CTA
+  const uint64_t want = a.all_queries ? (a.n_res + 3) / 4 : (a.n_res + 127) / 128;  // 4 warps per CTA, a query or 32 each
   const unsigned grid = (unsigned)(want < (uint64_t)nsm * 16 ? want : (uint64_t)nsm * 16);
   const bool epi = a.kp.epi_px >= 0.0;
   const uint32_t k = a.kp.top_k;
@@ -527,6 +592,34 @@ cudaError_t launch_match_fallback(const MatchArgs& a, cudaStream_t s) {
   else CHX_FB(32);
 #undef CHX_FB
   return cudaGetLastError();
+}
+
+// The per-pair schedule takes a warp per query (k_match_pair) unless a pair has more than 32,768 queries with more
+// than 2,048 lookup entries each: with a thread per query (k_match, direct) such a pair fills the GPU too and its
+// candidates come from shared memory.  us per pass over one pair, warps / threads: 2,000 x 2,000 features 20 / 43,
+// 8,000 36 / 88, 56,000 (1,312 entries) 396 / 476; short codes of 5 bits 8,000 80 / 243, 20,000 333 / 518, 40,000
+// (7,500 entries) 1,132 / 1,187, 56,000 2,077 / 1,616; of 2 bits 20,000 1,786 / 2,328, 40,000 6,233 / 5,550.
+bool match_pair_by_warps(const KParams& kp, uint32_t nA, uint32_t nB) {
+  return nA <= 32768u || ((uint64_t)kp.n_tables * nB >> kp.bits_per_table) <= 2048u;
+}
+
+cudaError_t launch_match_pair(const MatchArgs& a, uint32_t pair, const PairInfo& P, bool after, cudaStream_t s) {
+  if (P.nA == 0) return cudaSuccess;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((P.nA + 3) / 4);
+  cfg.blockDim = dim3(128);
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = after ? 1 : 0;
+  const bool epi = a.kp.epi_px >= 0.0;
+  const uint32_t k = a.kp.top_k;
+#define CHX_MP(KC) \
+  (epi ? cudaLaunchKernelEx(&cfg, k_match_pair<KC, true>, a, pair, P) : cudaLaunchKernelEx(&cfg, k_match_pair<KC, false>, a, pair, P))
+  return k <= 4 ? CHX_MP(4) : k <= 8 ? CHX_MP(8) : k <= 10 ? CHX_MP(10) : k <= 16 ? CHX_MP(16) : CHX_MP(32);
+#undef CHX_MP
 }
 
 // ---------------------------------------------------------------------------

@@ -88,13 +88,20 @@ extern "C" int cashash_match_pair_noalloc(const cashash_params* p, const cashash
   if (epi && (!F_dev || !s->kpts)) return CASHASH_EINVAL;
   if ((reinterpret_cast<uintptr_t>(match_off) & 7) || (reinterpret_cast<uintptr_t>(matches) & 3))
     return CASHASH_EINVAL;
-  // candidate-image chunk index and sizes from the host offsets
+  // candidate-image chunk index, sizes and bucket-sorted tables (behind all chunks) from the host offsets
   uint32_t bchunk0 = 0;
+  uint64_t n_chunks = 0, bjoin = 0;
   for (uint32_t i = 0; i < s->n_images; ++i) {
     if (s->img_off[i + 1] < s->img_off[i] || s->img_off[i + 1] - s->img_off[i] > CASHASH_MAX_IMAGE)
       return CASHASH_EINVAL;
-    if (i < image_b) bchunk0 += (uint32_t)((s->img_off[i + 1] - s->img_off[i] + JC - 1) / JC);
+    const uint64_t n = s->img_off[i + 1] - s->img_off[i];
+    n_chunks += (n + JC - 1) / JC;
+    if (i < image_b) {
+      bchunk0 += (uint32_t)((n + JC - 1) / JC);
+      bjoin += p->n_tables * join_block(n);
+    }
   }
+  bjoin += (n_chunks ? n_chunks : 1) * chunk_bytes(p->n_tables);
   const uint64_t nA = s->img_off[image_a + 1] - s->img_off[image_a];
   const uint64_t nB = s->img_off[image_b + 1] - s->img_off[image_b];
   if (nA > CASHASH_NOALLOC_MAX_QUERIES) return CASHASH_EINVAL;  // beyond the fixed scratch
@@ -123,6 +130,7 @@ extern "C" int cashash_match_pair_noalloc(const cashash_params* p, const cashash
   pi.nA = (uint32_t)nA;
   pi.nB = (uint32_t)nB;
   pi.bchunk0 = bchunk0;
+  pi.bjoin = bjoin;
   const uint32_t tile = (uint32_t)match_tile_size(p->top_k, 0);
   const uint32_t n_items = (uint32_t)((nA + tile - 1) / tile);
   if (n_items > CASHASH_NOALLOC_MAX_QUERIES / 256) return CASHASH_EINVAL;
@@ -147,7 +155,9 @@ extern "C" int cashash_match_pair_noalloc(const cashash_params* p, const cashash
   a.pair_cnt = &sc->count;
   a.status = &sc->status;
   a.kp = kp;
-  if (launch_match(a, 0, n_items, stream) != cudaSuccess) return CASHASH_ECUDA;
+  if ((match_pair_by_warps(kp, pi.nA, pi.nB) ? launch_match_pair(a, 0, pi, false, stream)
+                                             : launch_match(a, 0, n_items, stream)) != cudaSuccess)
+    return CASHASH_ECUDA;
   if (launch_scan_counts(&sc->count, 1, match_off, cap, &sc->status, &sc->total, stream) != cudaSuccess)
     return CASHASH_ECUDA;
   if (launch_compact(&sc->pair, 1, sc->res, match_off, matches, cap, stream) != cudaSuccess) return CASHASH_ECUDA;
