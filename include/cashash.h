@@ -203,11 +203,11 @@ void cashash_plan_destroy(cashash_plan* plan);
  * match_off is still complete, nothing beyond cap is written and
  * cashash_sync_status() returns EOVERFLOW.  Asynchronous on `stream`.
  * With the persistent schedule all pairs are matched by one batched kernel:
- * by default a bucket join when every query image has at most about 50,000
- * features (at least 40,000 whatever the parameters), else a speculative
+ * by default a warp per query for at most three pairs of images of up to
+ * 65,535 features; else a bucket join when every query image has at most about
+ * 50,000 features (at least 40,000 whatever the parameters), else a speculative
  * per-query kernel (cashash_plan_autotune may choose otherwise); the launch
- * sequence
- * is captured once as a CUDA graph (per set of output pointers, F and
+ * sequence is captured once as a CUDA graph (per set of output pointers, F and
  * profiling setting) and replayed on `stream`; calls on the same plan must
  * not overlap.
  * Errors: EINVAL, ECUDA. */

@@ -98,6 +98,9 @@ struct cashash_plan {
   double* d_F2 = nullptr;              // mutual check with the band: F of every matched pair (F, then F^T)
   uint64_t cap_F2 = 0;
   int persistent = 0;
+  bool one_shot = false;               // made for one match on stream `up`: launched without a graph
+  cudaStream_t up = nullptr;
+  uint8_t* d_slab = nullptr;           // one allocation: pairs, tau, pair counts + item counters, results
   PairInfo* d_pairs = nullptr;
   uint2* d_items = nullptr;
   uint32_t n_items = 0;
@@ -667,13 +670,9 @@ int cashash_get_mean(cashash_ctx* c, double* mean_out) {
 void cashash_plan_destroy(cashash_plan* pl) {
   if (!pl) return;
   cudaDeviceSynchronize();
-  dfree(pl->d_pairs);
+  dfree(pl->d_slab);
   dfree(pl->d_items);
-  dfree(pl->d_res);
-  dfree(pl->d_pair_cnt);
-  dfree(pl->d_item_ctr);
   dfree(pl->d_queue);
-  dfree(pl->d_tau);
   dfree(pl->d_jhist);
   dfree(pl->d_jline);
   dfree(pl->d_F2);
@@ -683,6 +682,16 @@ void cashash_plan_destroy(cashash_plan* pl) {
 }
 
 namespace {
+
+// Uploads and clears of a plan: in order before its match, on the stream of that match where the plan is made for
+// one, else as a caller of cashash_plan_create expects, whatever stream follows.
+cudaError_t plan_upload(const cashash_plan* pl, void* d, const void* h, size_t n) {
+  return pl->one_shot ? cudaMemcpyAsync(d, h, n, cudaMemcpyHostToDevice, pl->up)
+                      : cudaMemcpy(d, h, n, cudaMemcpyHostToDevice);
+}
+cudaError_t plan_clear(const cashash_plan* pl, void* d, size_t n) {
+  return pl->one_shot ? cudaMemsetAsync(d, 0, n, pl->up) : cudaMemset(d, 0, n);
+}
 
 // Work items, grid and scratch of a plan for configuration t (persistent
 // schedule), or for the per-pair schedule.  Drops the captured graph.
@@ -750,10 +759,10 @@ int plan_configure(cashash_plan* pl, cashash_tuning t) {
   } else {
     return CASHASH_EINVAL;
   }
-  int st = grow(pl->d_items, pl->cap_items, std::max<uint64_t>(items.size(), 1));
+  int st = items.empty() ? CASHASH_OK : grow(pl->d_items, pl->cap_items, items.size());
   if (st == CASHASH_OK && pl->persistent) {
     const uint64_t q = join ? (uint64_t)grid * pl->na_max * JSEG : (uint64_t)grid * t.tile * QCAP;
-    st = grow(pl->d_queue, pl->cap_queue, std::max<uint64_t>(q, 1));
+    if (q) st = grow(pl->d_queue, pl->cap_queue, q);
   }
   if (st == CASHASH_OK && join && epi)
     st = grow(pl->d_jline, pl->cap_jline, std::max<uint64_t>((uint64_t)grid * jline_stride(pl->na_max), 1));
@@ -761,10 +770,10 @@ int plan_configure(cashash_plan* pl, cashash_tuning t) {
     uint64_t cap = 0;
     st = grow(pl->d_jhist, cap, std::max<uint64_t>((uint64_t)P * HBINS, 1));
     if (st == CASHASH_OK)
-      st = cuda_err(cudaMemset(pl->d_jhist, 0, sizeof(uint32_t) * std::max<uint64_t>((uint64_t)P * HBINS, 1)));
+      st = cuda_err(plan_clear(pl, pl->d_jhist, sizeof(uint32_t) * std::max<uint64_t>((uint64_t)P * HBINS, 1)));
   }
   if (st == CASHASH_OK && !items.empty())
-    st = cuda_err(cudaMemcpy(pl->d_items, items.data(), sizeof(uint2) * items.size(), cudaMemcpyHostToDevice));
+    st = cuda_err(plan_upload(pl, pl->d_items, items.data(), sizeof(uint2) * items.size()));
   if (st != CASHASH_OK) return st;
   pl->n_items = (uint32_t)items.size();
   pl->join = join;
@@ -775,10 +784,20 @@ int plan_configure(cashash_plan* pl, cashash_tuning t) {
   return CASHASH_OK;
 }
 
-}  // namespace
+// Plans of at most three pairs take a warp per query by default: even clusters of 8 CTAs leave the join 24 of 304,
+// and its pass has a calibration and a fallback.  us per pass, join / warps: 1 pair of 1,000 x 1,000 features
+// 56 / 12, 8,000 160 / 35, 20,000 520 / 93, 40,000 1,523 / 261; 5-bit short codes 8,000 886 / 80; 3 pairs of 1,000
+// 57 / 14, 4,000 86 / 31.  (Images past 65,535 features, whose tables another kernel builds, were not measured.)
+constexpr uint32_t FEW_PAIRS = 3, FEW_FEATURES = 65535;
+bool plan_few(const cashash_plan* pl) {
+  if (pl->P == 0 || pl->P > FEW_PAIRS) return false;
+  for (const PairInfo& i : pl->info)
+    if (i.nA > FEW_FEATURES || i.nB > FEW_FEATURES) return false;
+  return join_grid(pl->ctx->kp, pl->na_max, pl->P, 0) != 0;
+}
 
-int cashash_plan_create(cashash_ctx* c, const cashash_set* s, const uint32_t* pairs_host, uint32_t P,
-                        cashash_plan** out) {
+int plan_create(cashash_ctx* c, const cashash_set* s, const uint32_t* pairs_host, uint32_t P, bool one_shot,
+                cudaStream_t stream, cashash_plan** out) {
   if (!c || !out || !set_ok(s, nullptr) || (P > 0 && !pairs_host)) return CASHASH_EINVAL;
   *out = nullptr;
   if (c->p.epi_px >= 0.0 && s->n_features > 0 && !s->kpts) return CASHASH_EINVAL;
@@ -805,6 +824,8 @@ int cashash_plan_create(cashash_ctx* c, const cashash_set* s, const uint32_t* pa
     pairs_host = pairs_int.data();
   }
   pl->ctx = c;
+  pl->one_shot = one_shot;
+  pl->up = stream;
   pl->P = P;
   pl->P_out = P_out;
   pl->persistent = c->p.schedule == CASHASH_SCHED_PERSISTENT;
@@ -846,25 +867,26 @@ int cashash_plan_create(cashash_ctx* c, const cashash_set* s, const uint32_t* pa
   pl->set.img_off = pl->img_off_h.data();
   pl->first.assign(P, 0);
   pl->count.assign(P, 0);
+  auto up = [](uint64_t n) { return (n + 255) / 256 * 256; };
+  const uint64_t o_tau = up(sizeof(PairInfo) * std::max<uint64_t>(P, 1)), o_cnt = o_tau + up(4 * std::max<uint64_t>(P, 1)),
+                 o_res = o_cnt + up(12 * (uint64_t)P + 12);
   uint64_t cap = 0;
-  int st = grow(pl->d_pairs, cap, std::max<uint64_t>(P, 1));
-  cap = 0;
-  if (st == CASHASH_OK) st = grow(pl->d_res, cap, std::max<uint64_t>(qbase, 1));
+  int st = grow(pl->d_slab, cap, o_res + 4 * std::max<uint64_t>(qbase, 1));
+  if (st == CASHASH_OK) {
+    pl->d_pairs = reinterpret_cast<PairInfo*>(pl->d_slab);
+    pl->d_tau = reinterpret_cast<uint32_t*>(pl->d_slab + o_tau);
+    pl->d_pair_cnt = reinterpret_cast<unsigned long long*>(pl->d_slab + o_cnt);  // [P], cleared with
+    pl->d_item_ctr = reinterpret_cast<unsigned int*>(pl->d_pair_cnt + P);        // ... [P + 1] in one go
+    pl->d_res = reinterpret_cast<uint32_t*>(pl->d_slab + o_res);
+    st = cuda_err(plan_clear(pl, pl->d_tau, sizeof(uint32_t) * std::max<uint64_t>(P, 1)));
+  }
   if (st == CASHASH_OK && P != P_out && c->p.epi_px >= 0.0)
     st = grow(pl->d_F2, pl->cap_F2, std::max<uint64_t>(9ull * P, 1));
-  cap = 0;
-  if (st == CASHASH_OK) st = grow(pl->d_pair_cnt, cap, std::max<uint64_t>(P, 1));
-  cap = 0;
-  if (st == CASHASH_OK) st = grow(pl->d_item_ctr, cap, (uint64_t)P + 1);
-  cap = 0;
-  if (st == CASHASH_OK) st = grow(pl->d_tau, cap, std::max<uint64_t>(P, 1));
-  if (st == CASHASH_OK) st = cuda_err(cudaMemset(pl->d_tau, 0, sizeof(uint32_t) * std::max<uint64_t>(P, 1)));
-  if (st == CASHASH_OK && P)
-    st = cuda_err(cudaMemcpy(pl->d_pairs, info.data(), sizeof(PairInfo) * P, cudaMemcpyHostToDevice));
+  if (st == CASHASH_OK && P) st = cuda_err(plan_upload(pl, pl->d_pairs, info.data(), sizeof(PairInfo) * P));
   if (st == CASHASH_OK) {
     if (pl->persistent) {
-      cashash_tuning t{};  // the join when it applies, else the per-query kernel
-      t.kernel = CASHASH_KERNEL_JOIN;
+      cashash_tuning t{};  // a warp per query for a few pairs, the join when it applies, else the per-query kernel
+      t.kernel = plan_few(pl) ? CASHASH_KERNEL_WARP : CASHASH_KERNEL_JOIN;
       t.tile = 4;
       st = plan_configure(pl, t);
       if (st == CASHASH_ENOTSUP) {
@@ -884,6 +906,13 @@ int cashash_plan_create(cashash_ctx* c, const cashash_set* s, const uint32_t* pa
   return CASHASH_OK;
 }
 
+}  // namespace
+
+int cashash_plan_create(cashash_ctx* c, const cashash_set* s, const uint32_t* pairs_host, uint32_t P,
+                        cashash_plan** out) {
+  return plan_create(c, s, pairs_host, P, false, nullptr, out);
+}
+
 namespace {
 
 // Enqueues the matching sequence of a plan on `stream`: counter resets, the
@@ -893,7 +922,7 @@ int enqueue_match(cashash_ctx* c, cashash_plan* pl, const double* F_dev, uint64_
                   uint64_t cap, cudaStream_t stream, bool capturing) {
   const uint32_t P = pl->P;
   const bool mutual = pl->P_out != pl->P;
-  if (P) CK(cudaMemsetAsync(pl->d_pair_cnt, 0, sizeof(unsigned long long) * P, stream));
+  CK(cudaMemsetAsync(pl->d_pair_cnt, 0, 12 * (size_t)P + 4, stream));  // and the item counters behind them
   if (mutual && c->p.epi_px >= 0.0 && F_dev) {  // F of the reverse pairs: transposed
     CK(launch_mutual_F(F_dev, pl->P_out, pl->d_F2, stream));
     F_dev = pl->d_F2;
@@ -923,7 +952,6 @@ int enqueue_match(cashash_ctx* c, cashash_plan* pl, const double* F_dev, uint64_
   a.jline = pl->d_jline;
   a.na_max = pl->na_max;
   a.kp = c->kp;
-  CK(cudaMemsetAsync(pl->d_item_ctr, 0, sizeof(unsigned int) * ((size_t)P + 1), stream));
   if (pl->persistent) {
     a.items = pl->d_items;
     a.n_items = pl->n_items;
@@ -992,7 +1020,7 @@ int cashash_match_plan(cashash_ctx* c, cashash_plan* pl, const double* F_dev, ui
   CK(cudaSetDevice(c->device));
   c->ev_used[CASHASH_STAGE_MATCH] = c->ev_used[CASHASH_STAGE_COMPACT] = 0;
   c->ev_used[CASHASH_STAGE_CALIBRATE] = c->ev_used[CASHASH_STAGE_FALLBACK] = 0;
-  if (pl->persistent) {
+  if (pl->persistent && !pl->one_shot) {
     const bool same = pl->gexec && pl->g_F == F_dev && pl->g_moff == match_off && pl->g_mt == matches &&
                       pl->g_cap == cap && pl->g_prof == c->profiling;
     if (!same) {
@@ -1223,7 +1251,7 @@ int cashash_match_pairs(cashash_ctx* c, const cashash_set* s, const uint32_t* pa
                         const double* F_dev, uint64_t* match_off, uint32_t* matches, uint64_t cap,
                         cashash_stream_t stream) {
   cashash_plan* pl = nullptr;
-  int st = cashash_plan_create(c, s, pairs_host, P, &pl);
+  int st = plan_create_once(c, s, pairs_host, P, reinterpret_cast<cudaStream_t>(stream), &pl);
   if (st != CASHASH_OK) return st;
   st = cashash_match_plan(c, pl, F_dev, match_off, matches, cap, stream);
   if (st == CASHASH_OK) st = cuda_err(cudaStreamSynchronize(reinterpret_cast<cudaStream_t>(stream)));
@@ -1460,3 +1488,8 @@ int cashash_run_host(cashash_ctx* c, const uint8_t* desc_host, const uint64_t* i
 }
 
 }  // extern "C"
+
+int chx::plan_create_once(cashash_ctx* c, const cashash_set* s, const uint32_t* pairs_host, uint32_t P,
+                          cudaStream_t stream, cashash_plan** out) {
+  return plan_create(c, s, pairs_host, P, true, stream, out);
+}

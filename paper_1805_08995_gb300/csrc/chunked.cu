@@ -79,7 +79,7 @@ extern "C" int cashash_match_chunked(cashash_ctx* c, const cashash_set* s, const
     int st = buf.reserve((uint64_t)count + 1, std::max<uint64_t>(cap, 1));
     if (st != CASHASH_OK) return st;
     cashash_plan* pl = nullptr;
-    st = cashash_plan_create(c, s, pr, count, &pl);
+    st = plan_create_once(c, s, pr, count, stream, &pl);
     if (st != CASHASH_OK) return st;
     cashash_tuning want{}, cur{};
     if (cashash_get_host_tuning(c, &want) == CASHASH_OK && want.kernel != 0 &&

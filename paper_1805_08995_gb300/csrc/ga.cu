@@ -816,10 +816,11 @@ extern "C" int cashash_ga_stage1(cashash_ctx* ctx, const cashash_set* set, const
   if ((st = cashash_build_codes(ctx, &S, mean_host, stream_)) != CASHASH_OK) return st;
   if (P == 0) return err_of(cudaStreamSynchronize(s));
   cashash_plan* pl = nullptr;
-  if ((st = cashash_plan_create(ctx, &S, pairs_host, P, &pl)) != CASHASH_OK) return st;
+  if ((st = plan_create_once(ctx, &S, pairs_host, P, s, &pl)) != CASHASH_OK) return st;
   cashash_tuning tu{};
   if (cashash_plan_get_tuning(pl, &tu) == CASHASH_OK && tu.kernel != 0) {  // batched plans only
     uint32_t want = gp->kernel;
+    if (want == 0 && tu.kernel == CASHASH_KERNEL_WARP) want = tu.kernel;  // a few pairs
     if (want == 0) want = N < 4096ull * std::max<uint32_t>(n_images, 1) ? CASHASH_KERNEL_QUERY : CASHASH_KERNEL_JOIN;
     if (want != tu.kernel) {
       cashash_tuning t2{};

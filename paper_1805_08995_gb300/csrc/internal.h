@@ -238,6 +238,11 @@ __device__ __forceinline__ bool epi_keep_fast(const EpiQ& e, float2 pc) {
 // finite band width), else 0.
 int params_ok(const cashash_params* p);
 
+// A plan for one match on `stream` (cashash_plan_create otherwise): its uploads are in order on that stream, and
+// the match is launched without a graph, which only repays its capture when replayed.
+int plan_create_once(cashash_ctx* c, const cashash_set* s, const uint32_t* pairs_host, uint32_t P, cudaStream_t stream,
+                     cashash_plan** out);
+
 // ---- launchers (return cudaError_t of the launch) ----
 // Column sums of n descriptors into sums[128] (zeroed first unless add).
 cudaError_t launch_colsum(const uint8_t* desc, uint64_t n, unsigned long long* sums, cudaStream_t s,

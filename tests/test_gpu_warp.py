@@ -61,3 +61,50 @@ def test_per_pair_largest_pairs(ch, orc):  # noqa: F811
     pk = dict(bits_per_table=1, n_tables=2)  # 2,100 candidates per query
     ctx, *_ = _compare(ch, orc, s, np.array([[0, 2], [1, 2], [2, 2], [2, 1]], np.uint32), pk)
     ctx.close()
+
+
+@pytest.mark.parametrize("flags", [0, 1])
+def test_plans_of_a_few_pairs(ch, orc, flags):  # noqa: F811
+    """One to four pairs around the rule that gives a few pairs a warp per query: kept plans under every kernel, and
+    calls that make their plan for one match, on a stream of their own that nothing orders with the others."""
+    sizes = [900, 0, 1, 2500]
+    s = synth.random_set(618, sizes)
+    pk = dict(schedule=1, flags=flags)
+    p = ch.cashash_default_params(**pk)
+    ctx = ch.cashash_create(p, s.R)
+    ds = ch.DeviceSet(p, s.img_off, s.desc, s.kpts)
+    ch.cashash_build_codes(ctx, ds)
+    torch.cuda.synchronize()
+    po = oparams(orc, pk)
+    mu, codes, buckets = oracle_codes(orc, s.desc, s.R, po)
+    side = torch.cuda.Stream()
+    for pairs in ([[0, 3]], [[3, 0], [0, 1]], [[0, 3], [1, 1], [2, 3]], [[0, 3], [3, 0], [3, 3], [2, 0]]):
+        pairs = np.array(pairs, np.uint32)
+        eoff, emt = orc.match_pairs(s.desc, s.img_off, codes, buckets, pairs, po)
+        cap = int(s.sizes()[pairs[:, 0]].sum())
+        moff = torch.zeros(len(pairs) + 1, dtype=torch.int64, device="cuda")
+        mt = torch.zeros((cap, 2), dtype=torch.int32, device="cuda")
+
+        def check():
+            assert ch.cashash_sync_status(ctx) == ch.CASHASH_OK
+            off = moff.cpu().numpy().astype(np.uint64)
+            assert np.array_equal(off, eoff)
+            assert np.array_equal(mt[:int(off[-1])].cpu().numpy().view(np.uint32), emt)
+            moff.zero_()
+            mt.zero_()
+            torch.cuda.synchronize()
+
+        torch.cuda.synchronize()
+        for _ in range(3):
+            ch.cashash_match_pairs(ctx, ds, pairs, moff, mt, cap, stream=side.cuda_stream)
+            check()
+        plan = ch.cashash_plan_create(ctx, ds, pairs)
+        few = len(pairs) * (1 + flags) <= 3
+        assert ch.cashash_plan_get_tuning(plan)["kernel"] == (ch.CASHASH_KERNEL_WARP if few else ch.CASHASH_KERNEL_JOIN)
+        for kernel in (0, ch.CASHASH_KERNEL_JOIN, ch.CASHASH_KERNEL_QUERY, ch.CASHASH_KERNEL_WARP, 0):
+            if kernel:
+                ch.cashash_plan_set_tuning(plan, kernel, 0, 0)
+            ch.cashash_match_plan(ctx, plan, moff, mt, cap)
+            check()
+        plan.close()
+    ctx.close()
