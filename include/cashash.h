@@ -93,7 +93,8 @@ typedef struct {
   uint32_t ratio_den;
   uint32_t tau;             /* Sec. 6 threshold: candidates with Hamming > tau are dropped;
                                tau >= code_bits turns it off [code_bits] */
-  uint32_t precision;       /* CASHASH_FP32 (CUDA-core projection) or CASHASH_BF16 (tensor cores) */
+  uint32_t precision;       /* CASHASH_FP32 or CASHASH_BF16: both run the tensor-core projection with 31-bit
+                               weights; codes never depended on it */
   uint32_t schedule;        /* CASHASH_SCHED_PER_PAIR (one launch per pair) or
                                CASHASH_SCHED_PERSISTENT (one launch over the whole pair list) */
   uint32_t flags;           /* CASHASH_FLAG_* below, ORed [0] */
@@ -161,8 +162,8 @@ int cashash_build_codes(cashash_ctx* ctx, const cashash_set* set, const double* 
 
 /* Diagnostic of the rounding bound of the projection (Sec. 5.1; not needed
  * for matching).  For features [first, first + count) of `set`, runs the
- * context's projection form (precision FP32 or BF16) with the centre and row
- * constants of the last cashash_build_codes on this context, and writes, row-
+ * projection with the centre and row constants of the last
+ * cashash_build_codes on this context, and writes, row-
  * major [count][rows] with rows = code_bits + n_tables * bits_per_table:
  *   approx: the FP32 approximation v~_b - c_b of each projection
  *           v_b = sum_j R_bj (x_j - mu_j), as the kernel computed it;

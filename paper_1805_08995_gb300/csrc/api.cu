@@ -48,9 +48,9 @@ struct cashash_ctx {
   uint32_t rows = 0;
   double* d_R = nullptr;        // [rows][128]
   double* d_nrmR = nullptr;     // [rows]
-  float* d_R32T = nullptr;      // [128][192] FP32 R, transposed, zero padded
-  void* d_Rbf = nullptr;        // BF16 form operands: R hi and lo, core-matrix layout
-  uint32_t np_tc = 0;           // BF16 form: rows padded to a multiple of 16
+  int* d_expo = nullptr;        // [rows] exponents s_b that scale the rows of R
+  void* d_Rs = nullptr;         // projection operands: hi, mid and lo of the scaled R, core-matrix layout
+  uint32_t np_tc = 0;           // rows padded to a multiple of 16
   double* d_mu = nullptr;       // [128]
   RowConst* d_rc = nullptr;     // [192]
   unsigned long long* d_colsum = nullptr;  // [128]
@@ -173,6 +173,14 @@ int cuda_err(cudaError_t e) {
   } while (0)
 
 
+// The f16 bits of k * 2^e, exact: |k| <= 2048, e >= -14.
+uint16_t f16_of_int(int k, int e) {
+  if (k == 0) return 0u;
+  const uint32_t a = (uint32_t)(k < 0 ? -k : k);
+  const int t = 31 - __builtin_clz(a);  // a = 1.xxx * 2^t
+  return (uint16_t)((k < 0 ? 0x8000u : 0u) | (uint32_t)(t + e + 15) << 10 | ((a << 11 >> (t + 1)) & 0x3FFu));
+}
+
 template <class T>
 int grow(T*& ptr, uint64_t& cap, uint64_t need) {
   if (need <= cap && ptr) return CASHASH_OK;
@@ -196,30 +204,6 @@ template <class T>
 void dfree(T*& ptr) {
   if (ptr) cudaFree(ptr);
   ptr = nullptr;
-}
-
-// Round-to-nearest-even of a double to bfloat16 (8-bit significand), bits.
-uint16_t bf16_rn(double x) {
-  if (x == 0.0 || !std::isfinite(x)) return std::signbit(x) ? 0x8000u : 0u;
-  int e = 0;
-  const double m = std::frexp(std::fabs(x), &e);  // |x| = m 2^e, m in [0.5, 1)
-  double M = std::nearbyint(std::ldexp(m, 8));     // 8 significant bits, ties to even
-  if (M == 256.0) {
-    M = 128.0;
-    e += 1;
-  }
-  const float v = (float)std::ldexp(M, e - 8);     // exact: at most 8 significant bits
-  uint32_t u;
-  std::memcpy(&u, &v, sizeof u);
-  if (x < 0) u |= 0x80000000u;
-  return (uint16_t)(u >> 16);
-}
-
-double bf16_to_double(uint16_t h) {
-  const uint32_t u = (uint32_t)h << 16;
-  float f;
-  std::memcpy(&f, &u, sizeof f);
-  return (double)f;
 }
 
 // Validates a set; returns number of lookup-table chunks through *n_chunks.
@@ -365,21 +349,15 @@ int build_codes_impl(cashash_ctx* c, const cashash_set* s, const double* mean_ho
       } else if (!sums_ready) {
         CK(launch_colsum(s->desc, n, c->d_colsum, st));
       }
-      // bound factor on ||R_b|| ||x||: FP32 FMA chains (2^-16), BF16 tensor cores (2^-15)
-      const float alpha_scale = c->p.precision == CASHASH_BF16 ? 0x1p-15f : 0x1p-16f;
-      CK(launch_row_consts(c->d_colsum, n, mean_host ? 1 : 0, c->d_mu, c->d_R, c->d_nrmR, c->rows, alpha_scale,
-                           c->d_rc, st));
+      CK(launch_row_consts(c->d_colsum, n, mean_host ? 1 : 0, c->d_mu, c->d_R, c->d_nrmR, c->d_expo, c->rows, c->d_rc,
+                           st));
       CK(cudaMemsetAsync(c->d_cnt, 0, 2 * sizeof(unsigned long long), st));
     }
     if (n) {
       {
         StageTimer tm(c, CASHASH_STAGE_PROJECT, st, capturing);
-        if (c->p.precision == CASHASH_BF16)
-          CK(launch_project_bf16(s->desc, n, c->d_Rbf, c->np_tc, c->d_rc, c->kp, s->codes, s->buckets, s->sqnorm,
-                                 c->d_flagmask, c->d_flaglist, c->d_cnt + 0, c->d_status, st));
-        else
-          CK(launch_project_fp32(s->desc, n, c->d_R32T, c->d_rc, c->kp, s->codes, s->buckets, s->sqnorm,
-                                 c->d_flagmask, c->d_flaglist, c->d_cnt + 0, st));
+        CK(launch_project(s->desc, n, c->d_Rs, c->np_tc, c->d_rc, c->kp, s->codes, s->buckets, s->sqnorm,
+                          c->d_flagmask, c->d_flaglist, c->d_cnt + 0, c->d_status, st));
       }
       {
         StageTimer tm(c, CASHASH_STAGE_REEVAL, st, capturing);
@@ -517,7 +495,7 @@ void cashash_destroy(cashash_ctx* c) {
   if (c->bg_stream) cudaStreamDestroy(c->bg_stream);
   if (h.copy) cudaStreamDestroy(h.copy);
   if (h.comp) cudaStreamDestroy(h.comp);
-  dfree(c->d_R); dfree(c->d_nrmR); dfree(c->d_R32T); dfree(c->d_Rbf); dfree(c->d_mu); dfree(c->d_rc);
+  dfree(c->d_R); dfree(c->d_nrmR); dfree(c->d_expo); dfree(c->d_Rs); dfree(c->d_mu); dfree(c->d_rc);
   dfree(c->d_colsum); dfree(c->d_cnt); dfree(c->d_status); dfree(c->d_flagmask); dfree(c->d_flaglist);
   dfree(c->d_chunk_feat0); dfree(c->d_chunk_len);
   dfree(c->d_img_f0); dfree(c->d_img_n); dfree(c->d_img_join);
@@ -549,14 +527,12 @@ int cashash_create(cashash_ctx** out, const cashash_params* p, const double* R_h
   c->kp.flags = p->flags;
   int st = cuda_err(cudaGetDevice(&c->device));
   if (st == CASHASH_OK) st = cuda_err(cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, c->device));
-  // host-side constants: FP32 transposed copy of R and row norms (rounded up)
-  std::vector<float> r32t((size_t)DIM * 192, 0.f);
+  // host-side constants: row norms (rounded up) and the split of R
   std::vector<double> nrm(rows, 0.0);
   for (uint32_t b = 0; b < rows; ++b) {
     long double s = 0.0L;
     for (int j = 0; j < DIM; ++j) {
       const double v = R_host[(size_t)b * DIM + j];
-      r32t[(size_t)j * 192 + b] = (float)v;
       s += (long double)v * (long double)v;
     }
     nrm[b] = (double)sqrtl(s) * (1.0 + 1e-12);
@@ -566,7 +542,7 @@ int cashash_create(cashash_ctx** out, const cashash_params* p, const double* R_h
   cap = 0;
   if (st == CASHASH_OK) st = grow(c->d_nrmR, cap, rows);
   cap = 0;
-  if (st == CASHASH_OK) st = grow(c->d_R32T, cap, (uint64_t)DIM * 192);
+  if (st == CASHASH_OK) st = grow(c->d_expo, cap, rows);
   cap = 0;
   if (st == CASHASH_OK) st = grow(c->d_mu, cap, DIM);
   cap = 0;
@@ -579,29 +555,39 @@ int cashash_create(cashash_ctx** out, const cashash_params* p, const double* R_h
   if (st == CASHASH_OK) st = grow(c->d_status, cap, 1);
   if (st == CASHASH_OK) st = cuda_err(cudaMemcpy(c->d_R, R_host, sizeof(double) * rows * DIM, cudaMemcpyHostToDevice));
   if (st == CASHASH_OK) st = cuda_err(cudaMemcpy(c->d_nrmR, nrm.data(), sizeof(double) * rows, cudaMemcpyHostToDevice));
-  if (st == CASHASH_OK)
-    st = cuda_err(cudaMemcpy(c->d_R32T, r32t.data(), sizeof(float) * r32t.size(), cudaMemcpyHostToDevice));
-  if (st == CASHASH_OK && p->precision == CASHASH_BF16) {
-    // R = hi + lo + r with hi = bf16(R), lo = bf16(R - hi) (R - hi is exact by Sterbenz), |r| <= 2^-16 |R|;
-    // laid out as K-major core matrices: (row group, k group) at ((r8 * 16 + k8) * 64) elements
+  if (st == CASHASH_OK) {
+    // the three f16 terms of the scaled rows (project_tc.cu), each laid out as K-major core matrices: (row group,
+    // k group) at ((r8 * 16 + k8) * 64) elements
     const uint32_t NP = (rows + 15) / 16 * 16;
     c->np_tc = NP;
-    std::vector<uint16_t> hb((size_t)2 * NP * DIM, 0);
-    for (uint32_t b = 0; b < rows; ++b)
-      for (int j = 0; j < DIM; ++j) {
-        const double v = R_host[(size_t)b * DIM + j];
-        const uint16_t hi = bf16_rn(v);
-        const uint16_t lo = bf16_rn(v - bf16_to_double(hi));
-        const size_t off = ((size_t)(b >> 3) * 16 + (j >> 3)) * 64 + (b & 7) * 8 + (j & 7);
-        hb[off] = hi;
-        hb[(size_t)NP * DIM + off] = lo;
+    std::vector<uint16_t> hb((size_t)3 * NP * DIM, 0);
+    std::vector<int> expo(rows, 0);
+    for (uint32_t b = 0; b < rows; ++b) {
+      double most = 0.0;
+      for (int j = 0; j < DIM; ++j) most = std::max(most, std::fabs(R_host[(size_t)b * DIM + j]));
+      int e = 0;
+      if (most > 0.0) {
+        std::frexp(most, &e);  // most in [2^(e - 1), 2^e)
+        e = std::min(9 - e, 999);
       }
+      expo[b] = e;
+      const double scale = std::ldexp(1.0, e);
+      for (int j = 0; j < DIM; ++j) {
+        const double r = R_host[(size_t)b * DIM + j] * scale, hi = std::rint(r), m = (r - hi) * 2048.0;
+        const double mid = std::rint(m), lo = std::rint((m - mid) * 2048.0);
+        const size_t off = ((size_t)(b >> 3) * 16 + (j >> 3)) * 64 + (b & 7) * 8 + (j & 7), part = (size_t)NP * DIM;
+        hb[off] = f16_of_int((int)hi, 0);
+        hb[part + off] = f16_of_int((int)mid, 0);
+        hb[2 * part + off] = f16_of_int((int)lo, -11);
+      }
+    }
+    st = cuda_err(cudaMemcpy(c->d_expo, expo.data(), sizeof(int) * rows, cudaMemcpyHostToDevice));
     cap = 0;
     uint16_t* d = nullptr;
-    st = grow(d, cap, hb.size());
-    c->d_Rbf = d;
+    if (st == CASHASH_OK) st = grow(d, cap, hb.size());
+    c->d_Rs = d;
     if (st == CASHASH_OK)
-      st = cuda_err(cudaMemcpy(c->d_Rbf, hb.data(), hb.size() * sizeof(uint16_t), cudaMemcpyHostToDevice));
+      st = cuda_err(cudaMemcpy(c->d_Rs, hb.data(), hb.size() * sizeof(uint16_t), cudaMemcpyHostToDevice));
   }
   if (st == CASHASH_OK) st = cuda_err(cudaMemset(c->d_cnt, 0, 8 * sizeof(unsigned long long)));
   if (st == CASHASH_OK) st = cuda_err(cudaMemset(c->d_status, 0, sizeof(uint32_t)));
@@ -641,14 +627,9 @@ int cashash_projection_bounds(cashash_ctx* c, const cashash_set* s, uint64_t fir
   if (st == CASHASH_OK) st = grow(cnt, c6, 2);
   if (st == CASHASH_OK) st = cuda_err(cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned long long), stream));
   const uint8_t* d = s->desc + first * DIM;
-  if (st == CASHASH_OK) {
-    if (c->p.precision == CASHASH_BF16)
-      st = cuda_err(launch_project_bf16(d, count, c->d_Rbf, c->np_tc, c->d_rc, c->kp, codes, bk, sqn, fm, fl, cnt,
-                                        c->d_status, stream, approx, bound));
-    else
-      st = cuda_err(launch_project_fp32(d, count, c->d_R32T, c->d_rc, c->kp, codes, bk, sqn, fm, fl, cnt, stream,
-                                        approx, bound));
-  }
+  if (st == CASHASH_OK)
+    st = cuda_err(launch_project(d, count, c->d_Rs, c->np_tc, c->d_rc, c->kp, codes, bk, sqn, fm, fl, cnt, c->d_status,
+                                 stream, approx, bound));
   if (st == CASHASH_OK) st = cuda_err(cudaStreamSynchronize(stream));
   dfree(codes);
   dfree(bk);

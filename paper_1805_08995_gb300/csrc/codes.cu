@@ -57,15 +57,15 @@ cudaError_t launch_colsum(const uint8_t* desc, uint64_t n, unsigned long long* s
 // Centre and per-row constants.  mu_j = S_j / N (one correctly rounded double
 // division).  c_b = sum_j R_bj mu_j is needed only by the approximation, so
 // its summation order is free; its error enters the bound.
-//   FP32 form bound (see the header comment of this file):
-//     |v~ - v_double| <= alpha_b ||x||_2 + beta_b,
-//     alpha_b = alpha_scale * ||R_b||_2,
-//     beta_b  = 2^-23 |c_b| + 2^-40 ||R_b||_2 (||mu||_2 + 1).
+//   |v~ - v_double| <= alpha_b ||x||_2 + beta_b (project_tc.cu), all in units of 2^-s_b,
+//     alpha_b = 2^-21 max(2^s ||R_b||_2, 256),
+//     beta_b  = 2^s (2^-23 |c_b| + 2^-40 ||R_b||_2 (||mu||_2 + 1)).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_row_consts(const unsigned long long* __restrict__ sums, uint64_t n,
                                                     int have_mean, double* __restrict__ mu,
                                                     const double* __restrict__ R, const double* __restrict__ nrmR,
-                                                    uint32_t rows, float alpha_scale, RowConst* __restrict__ rc) {
+                                                    const int* __restrict__ expo, uint32_t rows,
+                                                    RowConst* __restrict__ rc) {
   __shared__ double mu_s[DIM];
   __shared__ double nmu_s;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -99,157 +99,22 @@ __global__ void __launch_bounds__(256) k_row_consts(const unsigned long long* __
     for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xFFFFFFFFu, c, o);
     if (lane == 0) {
       RowConst r;
-      r.c32 = (float)c;
-      r.alpha = (float)(alpha_scale * nrmR[b] * (1.0 + 0x1p-20));
-      r.beta = (float)((0x1p-23 * fabs(c) + 0x1p-40 * nrmR[b] * (nmu_s + 1.0)) * (1.0 + 0x1p-20) + 0x1p-60);
-      r.pad = 0.f;
+      const int e = expo[b];
+      const double nr = scalbn(nrmR[b], e);
+      r.c32 = (float)scalbn(c, e);
+      r.alpha = (float)(0x1p-21 * fmax(nr, 256.0) * (1.0 + 0x1p-20));
+      r.beta = (float)((0x1p-23 * fabs(scalbn(c, e)) + 0x1p-40 * nr * (nmu_s + 1.0)) * (1.0 + 0x1p-20) + 0x1p-60);
+      r.pad = __int_as_float(e);
       rc[b] = r;
     }
   }
 }
 
 cudaError_t launch_row_consts(const unsigned long long* sums, uint64_t n, int have_mean, double* mu,
-                              const double* R, const double* nrmR, uint32_t rows, float alpha_scale,
-                              RowConst* rc, cudaStream_t s) {
+                              const double* R, const double* nrmR, const int* expo, uint32_t rows, RowConst* rc,
+                              cudaStream_t s) {
   // one warp per row, the rows spread over CTAs (each CTA derives the centre itself)
-  k_row_consts<<<(rows + 7) / 8, 256, 0, s>>>(sums, n, have_mean, mu, R, nrmR, rows, alpha_scale, rc);
-  return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------------------
-// FP32 CUDA-core projection.  Tile: 64 features x 192 rows per CTA of 256
-// threads; thread (fg, rg) owns features 4fg..4fg+3 and rows 12rg..12rg+11.
-// Each accumulator is one sequential FMA chain over j = 0..127, which the
-// bound alpha_scale = 2^-16 covers (gamma_256 for FP32 with margin).
-// ---------------------------------------------------------------------------
-constexpr int PT_F = 64;     // features per tile
-constexpr int PT_R = 192;    // rows per tile (padded)
-
-__global__ void __launch_bounds__(256, 1) k_project_fp32(const uint8_t* __restrict__ desc, uint64_t n,
-                                                         const float* __restrict__ R32T,
-                                                         const RowConst* __restrict__ rcg, KParams kp,
-                                                         uint32_t* __restrict__ codes, uint8_t* __restrict__ buckets,
-                                                         uint32_t* __restrict__ sqnorm,
-                                                         uint32_t* __restrict__ flagmask,
-                                                         uint32_t* __restrict__ flaglist,
-                                                         unsigned long long* __restrict__ nflag_feat,
-                                                         float* __restrict__ dbg_x, float* __restrict__ dbg_e) {
-  extern __shared__ __align__(16) float psm[];
-  float* Rs = psm;                       // [128][192]  R32 transposed (j-major)
-  float* xs = Rs + DIM * PT_R;           // [128][64]   x as float (j-major)
-  __shared__ RowConst rc[PT_R];
-  __shared__ float nx_s[PT_F];
-  __shared__ uint32_t sq_s[PT_F];
-  __shared__ uint32_t sbits[PT_F][6];
-  __shared__ uint32_t sflag[PT_F][6];
-
-  const int tid = threadIdx.x;
-  for (int i = tid; i < DIM * PT_R / 4; i += 256)
-    reinterpret_cast<float4*>(Rs)[i] = __ldg(reinterpret_cast<const float4*>(R32T) + i);
-  for (int i = tid; i < PT_R; i += 256) {
-    if ((uint32_t)i < kp.rows) rc[i] = rcg[i];
-    else { RowConst z; z.c32 = 0.f; z.alpha = 0.f; z.beta = 0.f; z.pad = 0.f; rc[i] = z; }
-  }
-  const int fg = tid & 15, rg = tid >> 4;
-  const uint64_t ntiles = (n + PT_F - 1) / PT_F;
-  for (uint64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const uint64_t f0 = tile * PT_F;
-    __syncthreads();
-    // load 64 descriptors: thread -> feature tid>>2, bytes 32*(tid&3) .. +31
-    {
-      const int fl = tid >> 2, qq = tid & 3;
-      const uint64_t f = f0 + fl;
-      uint4 v0 = make_uint4(0, 0, 0, 0), v1 = v0;
-      if (f < n) {
-        const uint4* row = reinterpret_cast<const uint4*>(desc + f * DIM) + 2 * qq;
-        v0 = __ldg(row);
-        v1 = __ldg(row + 1);
-      }
-      const uint32_t w[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
-      uint32_t sq = 0;
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        sq = __dp4a(w[k], w[k], sq);
-#pragma unroll
-        for (int b = 0; b < 4; ++b) xs[(32 * qq + 4 * k + b) * PT_F + fl] = (float)((w[k] >> (8 * b)) & 0xFFu);
-      }
-      sq += __shfl_xor_sync(0xFFFFFFFFu, sq, 1);
-      sq += __shfl_xor_sync(0xFFFFFFFFu, sq, 2);
-      if (qq == 0) {
-        sq_s[fl] = sq;
-        nx_s[fl] = sqrtf((float)sq);
-      }
-      if (tid < PT_F * 6) {
-        (&sbits[0][0])[tid] = 0u;
-        (&sflag[0][0])[tid] = 0u;
-      }
-      if (tid + 256 < PT_F * 6) {
-        (&sbits[0][0])[tid + 256] = 0u;
-        (&sflag[0][0])[tid + 256] = 0u;
-      }
-    }
-    __syncthreads();
-    float acc[4][12];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < 12; ++b) acc[a][b] = 0.f;
-#pragma unroll 4
-    for (int j = 0; j < DIM; ++j) {
-      const float4 xv = *reinterpret_cast<const float4*>(xs + j * PT_F + 4 * fg);
-      const float4 r0 = *reinterpret_cast<const float4*>(Rs + j * PT_R + 12 * rg);
-      const float4 r1 = *reinterpret_cast<const float4*>(Rs + j * PT_R + 12 * rg + 4);
-      const float4 r2 = *reinterpret_cast<const float4*>(Rs + j * PT_R + 12 * rg + 8);
-      const float xa[4] = {xv.x, xv.y, xv.z, xv.w};
-      const float ra[12] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w, r2.x, r2.y, r2.z, r2.w};
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 12; ++b) acc[a][b] = __fmaf_rn(ra[b], xa[a], acc[a][b]);
-    }
-    // signs, bound test, flags
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      const int fl = 4 * fg + a;
-      const float nx = nx_s[fl];
-#pragma unroll
-      for (int b = 0; b < 12; ++b) {
-        const int row = 12 * rg + b;
-        if ((uint32_t)row < kp.rows) {
-          const RowConst r = rc[row];
-          const float v = acc[a][b] - r.c32;
-          const float E = __fmaf_ru(r.alpha, nx, r.beta);
-          if (dbg_x && f0 + fl < n) {  // diagnostic of the bound (cashash_projection_bounds)
-            dbg_x[(f0 + fl) * kp.rows + row] = v;
-            dbg_e[(f0 + fl) * kp.rows + row] = E;
-          }
-          if (fabsf(v) <= E) atomicOr(&sflag[fl][row >> 5], 1u << (row & 31));
-          else if (v > 0.f) atomicOr(&sbits[fl][row >> 5], 1u << (row & 31));
-        }
-      }
-    }
-    __syncthreads();
-    if (tid < PT_F && f0 + tid < n)
-      write_feature(f0 + tid, sbits[tid], sflag[tid], sq_s[tid], kp, codes, buckets, sqnorm, flagmask, flaglist,
-                    nflag_feat);
-  }
-}
-
-cudaError_t launch_project_fp32(const uint8_t* desc, uint64_t n, const float* R32T, const RowConst* rc,
-                                const KParams& kp, uint32_t* codes, uint8_t* buckets, uint32_t* sqnorm,
-                                uint32_t* flagmask, uint32_t* flaglist, unsigned long long* nflag_feat,
-                                cudaStream_t s, float* dbg_x, float* dbg_e) {
-  if (n == 0) return cudaSuccess;
-  const size_t smem = (size_t)DIM * PT_R * 4 + (size_t)DIM * PT_F * 4;
-  cudaError_t e = cudaFuncSetAttribute(k_project_fp32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  int dev = 0, nsm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  const uint64_t ntiles = (n + PT_F - 1) / PT_F;
-  const int grid = (int)(ntiles < (uint64_t)nsm ? ntiles : (uint64_t)nsm);
-  k_project_fp32<<<grid, 256, smem, s>>>(desc, n, R32T, rc, kp, codes, buckets, sqnorm, flagmask, flaglist,
-                                         nflag_feat, dbg_x, dbg_e);
+  k_row_consts<<<(rows + 7) / 8, 256, 0, s>>>(sums, n, have_mean, mu, R, nrmR, expo, rows, rc);
   return cudaGetLastError();
 }
 

@@ -60,13 +60,13 @@ __host__ __device__ inline uint64_t jline_stride(uint64_t na_max) { return na_ma
 
 // Per-row constants of the projection (Sec. 5.1) derived from R and the centre.
 struct RowConst {
-  float c32;     // fl32(c_b), c_b = sum_j R_bj mu_j
-  float alpha;   // bound factor on ||x||_2 (FP32 form) or on ||x||_2 (BF16 form)
+  float c32;     // fl32(2^s_b c_b), c_b = sum_j R_bj mu_j
+  float alpha;   // bound factor on ||x||_2
   float beta;    // additive bound term
-  float pad;
+  float pad;     // the bits of s_b (all above in units of 2^-s_b)
 };
 
-constexpr int PT_ROWS_TC = 192;   // projection rows supported by the tensor-core form (padded to 16)
+constexpr int PT_ROWS_TC = 192;   // projection rows supported (padded to 16)
 
 #ifdef __CUDACC__
 // ---------------------------------------------------------------------------
@@ -83,9 +83,9 @@ __device__ __forceinline__ uint32_t extract_bits(const uint32_t* w, uint32_t pos
 }
 
 __device__ __forceinline__ void write_feature(uint64_t f, const uint32_t* bits, const uint32_t* flags,
-                                              uint32_t sq, const KParams& kp, uint32_t* __restrict__ codes,
-                                              uint8_t* __restrict__ buckets, uint32_t* __restrict__ sqnorm,
-                                              uint32_t* __restrict__ flagmask, uint32_t* __restrict__ flaglist,
+                                              const KParams& kp, uint32_t* __restrict__ codes,
+                                              uint8_t* __restrict__ buckets, uint32_t* __restrict__ flagmask,
+                                              uint32_t* __restrict__ flaglist,
                                               unsigned long long* __restrict__ nflag_feat) {
   uint4 c;
   c.x = bits[0];
@@ -101,7 +101,6 @@ __device__ __forceinline__ void write_feature(uint64_t f, const uint32_t* bits, 
   bb.x = b[0] | (b[1] << 8) | (b[2] << 16) | (b[3] << 24);
   bb.y = b[4] | (b[5] << 8) | (b[6] << 16) | (b[7] << 24);
   reinterpret_cast<uint2*>(buckets)[f] = bb;
-  sqnorm[f] = sq;
   const uint32_t any = flags[0] | flags[1] | flags[2] | flags[3] | flags[4] | flags[5];
   if (any) {
 #pragma unroll
@@ -248,16 +247,12 @@ int plan_create_once(cashash_ctx* c, const cashash_set* s, const uint32_t* pairs
 cudaError_t launch_colsum(const uint8_t* desc, uint64_t n, unsigned long long* sums, cudaStream_t s,
                           bool add = false);
 cudaError_t launch_row_consts(const unsigned long long* sums, uint64_t n, int have_mean, double* mu,
-                              const double* R, const double* nrmR, uint32_t rows, float alpha_scale,
-                              RowConst* rc, cudaStream_t s);
-cudaError_t launch_project_fp32(const uint8_t* desc, uint64_t n, const float* R32T, const RowConst* rc,
-                                const KParams& kp, uint32_t* codes, uint8_t* buckets, uint32_t* sqnorm,
-                                uint32_t* flagmask, uint32_t* flaglist, unsigned long long* nflag_feat,
-                                cudaStream_t s, float* dbg_x = nullptr, float* dbg_e = nullptr);
-cudaError_t launch_project_bf16(const uint8_t* desc, uint64_t n, const void* Rbf, uint32_t NP, const RowConst* rc,
-                                const KParams& kp, uint32_t* codes, uint8_t* buckets, uint32_t* sqnorm,
-                                uint32_t* flagmask, uint32_t* flaglist, unsigned long long* nflag_feat,
-                                uint32_t* status, cudaStream_t s, float* dbg_x = nullptr, float* dbg_e = nullptr);
+                              const double* R, const double* nrmR, const int* expo, uint32_t rows, RowConst* rc,
+                              cudaStream_t s);
+cudaError_t launch_project(const uint8_t* desc, uint64_t n, const void* Rs, uint32_t NP, const RowConst* rc,
+                           const KParams& kp, uint32_t* codes, uint8_t* buckets, uint32_t* sqnorm, uint32_t* flagmask,
+                           uint32_t* flaglist, unsigned long long* nflag_feat, uint32_t* status, cudaStream_t s,
+                           float* dbg_x = nullptr, float* dbg_e = nullptr);
 // (dbg_x, dbg_e: when non-null, [n][rows] FP32 approximation v~ - c and bound E of
 // every projection, for cashash_projection_bounds; null in the matching path.)
 cudaError_t launch_fix_fp64(const uint8_t* desc, const double* mu, const double* R, const KParams& kp,

@@ -1,106 +1,97 @@
-// BF16 tensor-core form of the projection of Sec. 5.1 (tcgen05 + TMEM, sm_103a).
+// Projection of Sec. 5.1 on tcgen05 tensor cores (sm_103a), for either precision setting.
 //
-// v_fb = sum_j R_bj x_fj - c_b is computed as a GEMM D[128 features x N rows]
-// = X (uint8 -> bf16, exact) times [Rhi | Rlo]^T, where Rhi = bf16(R) and
-// Rlo = bf16(R - Rhi) (both round-to-nearest, so |R - Rhi - Rlo| <= 2^-16 |R|),
-// accumulated in FP32 in tensor memory: K = 128 for Rhi, then K = 128 for Rlo
-// into the same accumulator.  Products of 8-bit integers and 8-bit-significand
-// bf16 values are exact in FP32.  For the accumulation the bound assumes a
-// pessimistic adder (every step truncates, no guard bits), which gives at most
-// 33 * 2^-23 * sum |terms| <= 2^-18 * 1.01 ||R_b|| ||x||; with the split
-// residual the error is below 1.26 * 2^-16 ||R_b|| ||x||, and the flag test
-// uses alpha = 2^-15 ||R_b||.  Everything under the bound is re-evaluated
-// exactly in double by k_fix_fp64, so the signs equal the double definition.
+// v_fb = sum_j R_bj x_fj - c_b.  Row b of R is scaled by 2^s_b so that its largest entry lies in (256, 512] (a row
+// of zeros or of numbers below 2^-990 may stay smaller) and split into three f16 terms:
+//   r = 2^s R_bj,  hi = rint(r),  mid = rint(2^11 (r - hi)),  lo = 2^-11 rint(2^22 (r - hi) - 2^11 mid),
+// integers (lo: multiples of 2^-11) of up to 10 bits and the sign each, so normal f16 numbers.
+// x, 0 .. 255, is exact in f16.  One accumulator takes X hi^T: integers of at most 128 * 255 * 512 < 2^24, exact in
+// FP32 in any order.  A second one takes X mid^T, then X lo^T, and enters at 2^-11.  Error of A + 2^-11 B - c
+// against 2^s v, in units of N = max(2^s ||R_b||, 256) ||x||:
+//   * the split: |r - hi - 2^-11 (mid + lo)| <= 2^-23, so at most 2^-23 sum x <= 2^-23 sqrt(128) ||x|| < 2^-27 N;
+//   * B with a pessimistic adder (every step truncates, no guard bits): 33 * 2^-23 sum x |mid + lo| with |mid| <=
+//     1024, at 2^-11 half of 33 * 2^-23 sqrt(128) ||x||, below 2^-23.4 N for a row with one large entry (for rows
+//     of normal numbers, N = 1900 ||x||, eight times less);
+//   * A + 2^-11 B rounded: 2^-24 N; minus c: 2^-24 (N + |c|), and c is rounded itself: beta has 2^-23 |c|.
+// The sum is below 2^-22.2 N; the flag test takes 2^-21 N plus beta (which has the rounding of the double sequence
+// too).  |v~| under the bound goes to k_fix_fp64, so the signs equal the double definition.
 //
-// Shared-memory operands use the canonical K-major layout without swizzle:
-// 8-row x 16-byte core matrices of 128 contiguous bytes; core matrix (r8, k8)
-// sits at (r8 * 16 + k8) * 128 bytes, so the leading-dimension offset (next
+// Before, the FP32 setting took CUDA-core FMA chains over 24-bit weights (bound 2^-16) and the other one a two-term
+// bf16 split (2^-15).  Against the doubles, over 60,000 features and 176 rows of normal numbers: error 1.9e-5 rms and
+// 1.7e-4 at most, where the FMA chains had 1.1e-4 and 1.5e-3 and the bf16 split 1.3e-3 and 6.6e-3; of 844,018
+// features 1,063 projections are re-evaluated, where it was 34,262 and 68,755.
+//
+// Shared-memory operands use the canonical K-major layout without swizzle: 8-row x 16-byte core matrices of 128
+// contiguous bytes; core matrix (r8, k8) sits at (r8 * 16 + k8) * 128 bytes, so the leading-dimension offset (next
 // core matrix along K) is 128 B and the stride offset (next 8 rows) is 2 KB.
 //
-// One CTA of 512 threads per SM, persistent over tiles of 128 features, with
-// two tiles in flight (two groups of 8 warps, each with its own A buffer,
-// TMEM accumulator and mbarrier; the R operands are shared).  Feature row r of
-// a group's tile is TMEM lane r; the two warps of a group that may access that
-// lane each convert half of the row's descriptor and read back half of its
-// accumulator columns with tcgen05.ld.  Every wait on an MMA mbarrier is
-// bounded; on timeout the group records an error and stops issuing work, and
-// the CTA still releases its tensor memory.
+// One CTA of 512 threads per SM, persistent over tiles of 128 features, two operand buffers.  The rows of R are
+// taken in two halves of up to 96 (one if all fit), each with its own two accumulators and mbarrier: while all warps
+// read one half back (feature row r is TMEM lane r; the four warps that may access a lane take 24 rows each), the
+// tensor cores work on the other.  773,191 features, 176 rows: 159 us (bf16 form 190); 321,454: 73 us (FP32 form 450).
+// Bound by the two barriers of a tile and by shared memory, which an MMA of 96 columns reads for 56 clocks where the
+// arithmetic takes 24 (issue 41 %, tensor pipe 28 % active).
+//
+// Every wait on an MMA mbarrier is bounded; on timeout the CTA records an error, waits (bounded) for what it still
+// has in flight, stops and releases its tensor memory.
 #include "tc_common.cuh"
 
 namespace chx {
 
 constexpr int TC_M = 128;
 constexpr int TC_K = 128;
-constexpr uint32_t TC_TMEM_COLS = 512;  // two accumulators of up to 192 columns
-constexpr int PT_THREADS = 512;          // two groups of 8 warps
-__device__ __forceinline__ uint32_t bf16x2_of_bytes(uint32_t w, int half) {
-  // two bytes of w (half 0: bytes 0,1; half 1: bytes 2,3) as bf16x2, exact
-  const float a = (float)((w >> (16 * half)) & 0xFFu);
-  const float b = (float)((w >> (16 * half + 8)) & 0xFFu);
+constexpr int TC_NH = 96;                // rows of R per half
+constexpr uint32_t TC_TMEM_COLS = 512;   // 2 halves x 2 accumulators x 96 columns
+constexpr int PT_THREADS = 512;
+
+// Two bytes of w (half 0: bytes 0, 1; half 1: bytes 2, 3) as f16x2, exact: 0x64bb is 1024 + bb.
+__device__ __forceinline__ uint32_t f16x2_of_bytes(uint32_t w, int half) {
+  const uint32_t x = __byte_perm(w, 0x64646464u, half ? 0x4342 : 0x4140);
   uint32_t r;
-  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
+  asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(0x64006400u));
   return r;
 }
 
-// Named barrier of one 256-thread feature group (ids 1 and 2; __syncthreads
-// uses 0).
-__device__ __forceinline__ void group_sync(uint32_t id) { asm volatile("bar.sync %0, 256;" ::"r"(id) : "memory"); }
-
-// The same barrier, returning whether any thread of the group passed x = true.
-__device__ __forceinline__ bool group_any(uint32_t id, bool x) {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\t"
-      "setp.ne.u32 q, %1, 0;\n\t"
-      "bar.red.or.pred p, %2, 256, q;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}\n"
-      : "=r"(r)
-      : "r"((uint32_t)x), "r"(id)
-      : "memory");
-  return r != 0;
+// 8 consecutive accumulator columns of this thread's TMEM lane (no wait).
+__device__ __forceinline__ void tmem_ld8_nowait(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
 }
 
-// Tile of 128 features: A = [16 row groups][16 k groups][128 B]; B = hi then
-// lo, each [NP/8 row groups][16 k groups][128 B].  Two groups of 8 warps work
-// on alternate tiles, each with its own A buffer, TMEM accumulator (columns
-// 0 and 256) and mbarrier, so one group's loads, MMAs and epilogue overlap the
-// other's.  In a group, warps 0-3 and 4-7 split every feature row: half h
-// converts descriptor bytes 64 h .. 64 h + 63 and reads accumulator columns
-// 96 h .. 96 h + 95 (rows 32 (w % 4) + lane of TMEM, the lanes warp w may
-// access); half 1 hands its code / flag words to half 0, which writes the
-// feature.
-__global__ void __launch_bounds__(PT_THREADS, 1) k_project_bf16(const uint8_t* __restrict__ desc, uint64_t n,
-                                                                const uint4* __restrict__ Rbf, uint32_t NP,
-                                                                const RowConst* __restrict__ rcg, KParams kp,
-                                                                uint32_t* __restrict__ codes,
-                                                                uint8_t* __restrict__ buckets,
-                                                                uint32_t* __restrict__ sqnorm,
-                                                                uint32_t* __restrict__ flagmask,
-                                                                uint32_t* __restrict__ flaglist,
-                                                                unsigned long long* __restrict__ nflag_feat,
-                                                                uint32_t* __restrict__ status,
-                                                                float* __restrict__ dbg_x,
-                                                                float* __restrict__ dbg_e) {
-  extern __shared__ __align__(1024) uint8_t tsm[];
+template <bool DBG>
+__global__ void __launch_bounds__(PT_THREADS, 1) k_project(const uint8_t* __restrict__ desc, uint64_t n,
+                                                           const uint4* __restrict__ Rs, uint32_t NP,
+                                                           const RowConst* __restrict__ rcg, KParams kp,
+                                                           uint32_t* __restrict__ codes,
+                                                           uint8_t* __restrict__ buckets,
+                                                           uint32_t* __restrict__ sqnorm,
+                                                           uint32_t* __restrict__ flagmask,
+                                                           uint32_t* __restrict__ flaglist,
+                                                           unsigned long long* __restrict__ nflag_feat,
+                                                           uint32_t* __restrict__ status,
+                                                           float* __restrict__ dbg_x, float* __restrict__ dbg_e) {
+  extern __shared__ __align__(128) uint8_t tsm[];
   __shared__ __align__(8) uint64_t s_mbar[2];
   __shared__ uint32_t s_tmem;
-  __shared__ RowConst rc[PT_ROWS_TC];
-  __shared__ uint32_t s_sq[2][2][TC_M];  // [group][half][row]: partial squared norms
-  __shared__ uint32_t s_hi[2][6][TC_M];  // [group][word][row]: code words 3..5, then flag words 3..5
+  __shared__ float4 rc[PT_ROWS_TC];            // c, alpha, beta
+  __shared__ float s_nx[2][TC_M];              // [tile parity][row]: ||x||
+  __shared__ uint32_t s_bits[2][8][TC_M];      // [tile parity][24 rows of R][row]: signs
+  __shared__ uint32_t s_flag[2][6][TC_M];      // [tile parity][word][row]: rows under the bound (zero in between)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int grp = warp >> 3, half = (warp >> 2) & 1, quarter = warp & 3;
-  const uint32_t r = (uint32_t)(quarter * 32 + lane);  // feature row in the tile = TMEM lane
-  const int leader = grp * 256;                        // issues the group's MMAs
-  uint8_t* As = tsm + grp * (TC_M * TC_K * 2);         // 32 KB per group
-  uint8_t* Bs = tsm + 2 * (TC_M * TC_K * 2);           // 2 x NP x 256 B
-  const uint32_t bbytes = NP * TC_K * 2;               // one of hi / lo
+  const int cg = warp >> 2;                                       // 24 of a half's 96 rows of R
+  const uint32_t r = (uint32_t)((warp & 3) * 32 + lane);          // feature row in the tile = TMEM lane
+  uint8_t* As = tsm;                                              // 2 x 32 KB
+  uint8_t* Bs = tsm + 2 * (TC_M * TC_K * 2);                      // hi, mid, lo: NP x 256 B each
+  const uint32_t bbytes = NP * TC_K * 2;
+  const int halves = NP > TC_NH ? 2 : 1;
 
-  // operands of R (hi and lo) and the row constants, once per CTA
-  for (uint32_t i = tid; i < 2 * bbytes / 16; i += PT_THREADS) reinterpret_cast<uint4*>(Bs)[i] = __ldg(Rbf + i);
+  for (uint32_t i = tid; i < 3 * bbytes / 16; i += PT_THREADS) reinterpret_cast<uint4*>(Bs)[i] = __ldg(Rs + i);
   for (int i = tid; i < PT_ROWS_TC; i += PT_THREADS) {
-    if ((uint32_t)i < kp.rows) rc[i] = rcg[i];
-    else { RowConst z; z.c32 = 0.f; z.alpha = 0.f; z.beta = 0.f; z.pad = 0.f; rc[i] = z; }
+    RowConst z{};
+    if ((uint32_t)i < kp.rows) z = rcg[i];
+    rc[i] = make_float4(z.c32, z.alpha, z.beta, 0.f);
   }
+  for (int i = tid; i < 2 * 6 * TC_M; i += PT_THREADS) (&s_flag[0][0][0])[i] = 0u;
   if (tid == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_mbar[0])) : "memory");
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_mbar[1])) : "memory");
@@ -112,130 +103,145 @@ __global__ void __launch_bounds__(PT_THREADS, 1) k_project_bf16(const uint8_t* _
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+
+  // 8 features x 4 quarter rows of 32 bytes per warp: conflict-free stores, whole descriptors per warp
+  const uint32_t lrow = (uint32_t)(warp * 8 + (lane & 7)), part = (uint32_t)lane >> 3;
+  const uint64_t ntiles = (n + TC_M - 1) / TC_M;
+  uint4 v[2];
+  auto load_tile = [&](uint64_t t) {
+    v[0] = v[1] = make_uint4(0u, 0u, 0u, 0u);
+    const uint64_t f = t * TC_M + lrow;
+    if (t < ntiles && f < n) {
+      const uint4* src = reinterpret_cast<const uint4*>(desc + f * DIM) + 2 * part;
+      v[0] = __ldg(src);
+      v[1] = __ldg(src + 1);
+    }
+  };
+  // the loaded bytes -> f16 operand rows of buffer b, the norms; sqnorm is written here
+  auto convert = [&](uint64_t t, uint32_t b) {
+    uint8_t* dst = As + b * (TC_M * TC_K * 2) + (lrow >> 3) * 2048 + (4 * part) * 128 + (lrow & 7) * 16;
+    uint32_t sq = 0;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const uint32_t w[4] = {v[c].x, v[c].y, v[c].z, v[c].w};
+#pragma unroll
+      for (int k = 0; k < 4; ++k) sq = __dp4a(w[k], w[k], sq);
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+        *reinterpret_cast<uint4*>(dst + (2 * c + k) * 128) =
+            make_uint4(f16x2_of_bytes(w[2 * k], 0), f16x2_of_bytes(w[2 * k], 1), f16x2_of_bytes(w[2 * k + 1], 0),
+                       f16x2_of_bytes(w[2 * k + 1], 1));
+    }
+    sq += __shfl_xor_sync(0xFFFFFFFFu, sq, 8);
+    sq += __shfl_xor_sync(0xFFFFFFFFu, sq, 16);
+    if (part == 0) {
+      s_nx[b][lrow] = __fsqrt_ru((float)sq);
+      if (t * TC_M + lrow < n) sqnorm[t * TC_M + lrow] = sq;
+    }
+  };
+  // the MMAs of half h of the tile in buffer b (one thread)
+  auto issue = [&](int h, uint32_t b) {
+    const uint32_t rows = h ? NP - TC_NH : min(NP, (uint32_t)TC_NH), idesc = tc_idesc_f16(TC_M, rows);
+    const uint32_t a0 = smem_u32(As) + b * (TC_M * TC_K * 2), b0 = smem_u32(Bs) + (uint32_t)h * (TC_NH / 8) * 2048u;
+    const uint32_t acc = s_tmem + (uint32_t)h * (2 * TC_NH);
+#pragma unroll
+    for (int p = 0; p < 3; ++p)
+#pragma unroll
+      for (int kk = 0; kk < TC_K / 16; ++kk)
+        tc_mma(acc + (p ? TC_NH : 0), tc_desc(a0 + kk * 256, 128, 2048), tc_desc(b0 + p * bbytes + kk * 256, 128, 2048),
+               idesc, (p == 2 || kk) ? 1u : 0u);
+    tc_commit(smem_u32(&s_mbar[h]));
+  };
+
+  uint64_t tile = blockIdx.x;
+  load_tile(tile);
+  convert(tile, 0);
+  load_tile(tile + gridDim.x);
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = s_tmem + (uint32_t)grp * 256u;  // this group's accumulator columns
-  const uint32_t mbar = smem_u32(&s_mbar[grp]);
-  const uint32_t bar_id = 1u + (uint32_t)grp;
-  const uint32_t idesc = tc_idesc(TC_M, NP);
-  const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
-
-  const uint64_t ntiles = (n + TC_M - 1) / TC_M;
-  const uint64_t stride = 2ull * gridDim.x;
-  uint64_t tile = 2ull * blockIdx.x + (uint64_t)grp;
-  // this thread's half row of a tile: 16-byte chunks 4 half .. 4 half + 3 (zeros beyond n)
-  uint4 v[4];
-  auto load_half = [&](uint64_t t) {
-    const uint64_t f = t * TC_M + r;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) v[c] = make_uint4(0u, 0u, 0u, 0u);
-    if (t < ntiles && f < n) {
-      const uint4* src = reinterpret_cast<const uint4*>(desc + f * DIM) + 4 * half;
-#pragma unroll
-      for (int c = 0; c < 4; ++c) v[c] = __ldg(src + c);
+  if (tid == 0)
+    for (int h = 0; h < halves; ++h) issue(h, 0);
+  const uint32_t lane_base = s_tmem + ((uint32_t)((warp & 3) * 32) << 16);
+  uint32_t phase = 0, b = 0;
+  for (; tile < ntiles; tile += gridDim.x, b ^= 1u, phase ^= 1u) {
+    const uint64_t f = tile * TC_M + r, next = tile + gridDim.x;
+    if (next < ntiles) {  // (its buffer's last MMAs were waited for in the previous round)
+      convert(next, b ^ 1u);
+      load_tile(next + gridDim.x);
     }
-  };
-  load_half(tile);
-  uint32_t phase = 0;
-  for (; tile < ntiles; tile += stride) {
-    const uint64_t f = tile * TC_M + r;
-    {  // descriptor bytes -> bf16 A rows, partial squared norm
-      uint8_t* rowbase = As + (r >> 3) * 2048 + (r & 7) * 16;
-      uint32_t sq = 0;
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {  // 16 bytes = 16 elements = two k groups
-        const int kc = 4 * half + c;
-        sq = __dp4a(v[c].x, v[c].x, sq);
-        sq = __dp4a(v[c].y, v[c].y, sq);
-        sq = __dp4a(v[c].z, v[c].z, sq);
-        sq = __dp4a(v[c].w, v[c].w, sq);
-        uint4 lo8, hi8;
-        lo8.x = bf16x2_of_bytes(v[c].x, 0);
-        lo8.y = bf16x2_of_bytes(v[c].x, 1);
-        lo8.z = bf16x2_of_bytes(v[c].y, 0);
-        lo8.w = bf16x2_of_bytes(v[c].y, 1);
-        hi8.x = bf16x2_of_bytes(v[c].z, 0);
-        hi8.y = bf16x2_of_bytes(v[c].z, 1);
-        hi8.z = bf16x2_of_bytes(v[c].w, 0);
-        hi8.w = bf16x2_of_bytes(v[c].w, 1);
-        *reinterpret_cast<uint4*>(rowbase + (2 * kc) * 128) = lo8;
-        *reinterpret_cast<uint4*>(rowbase + (2 * kc + 1) * 128) = hi8;
-      }
-      s_sq[grp][half][r] = sq;
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    group_sync(bar_id);
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (tid == leader) {
-      const uint32_t a0 = smem_u32(As), b0 = smem_u32(Bs);
-#pragma unroll
-      for (int part = 0; part < 2; ++part) {  // Rhi, then Rlo
-#pragma unroll
-        for (int kk = 0; kk < TC_K / 16; ++kk) {
-          const uint64_t ad = tc_desc(a0 + kk * 256, 128, 2048);
-          const uint64_t bd = tc_desc(b0 + part * bbytes + kk * 256, 128, 2048);
-          tc_mma(tmem, ad, bd, idesc, (part | kk) ? 1u : 0u);
-        }
-      }
-      tc_commit(mbar);
-    }
-    load_half(tile + stride);  // the next tile's bytes are in flight during the MMAs and the epilogue
-    const bool waited = mbar_wait(mbar, phase);
-    if (group_any(bar_id, !waited)) {  // never expected: record it, let in-flight MMAs drain, stop
-      if (tid == leader) atomicOr(status, DST_INDEX);
-      mbar_wait(mbar, phase);
-      break;
-    }
-    phase ^= 1u;
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    // epilogue: this thread's 96 accumulator columns, 16 at a time
-    const uint32_t sq = s_sq[grp][0][r] + s_sq[grp][1][r];
-    const float nx = sqrtf((float)sq);
-    uint32_t bits[3] = {0u, 0u, 0u}, flags[3] = {0u, 0u, 0u};  // rows 96 half + 32 k + bit
-#pragma unroll
-    for (int b = 0; b < 2; ++b) {  // three 16-column loads in flight
-      uint32_t r3[3][16];
+    const float nx = s_nx[b][r];
+    bool failed = false;
+    for (int h = 0; h < halves; ++h) {
+      const bool waited = mbar_wait(smem_u32(&s_mbar[h]), phase);
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t col = lane_base + (uint32_t)(h * 2 * TC_NH + cg * 24);
+      uint32_t hi[3][8], lo[3][8], pos = 0, out = 0;  // bit 23 - i: row i's sign, and whether it is outside the bound
 #pragma unroll
       for (int u = 0; u < 3; ++u) {
-        const uint32_t col = (uint32_t)(96 * half + (3 * b + u) * 16);
-        if (col < NP) tmem_ld16_nowait(tmem + lane_base + col, r3[u]);
+        tmem_ld8_nowait(col + u * 8, hi[u]);
+        tmem_ld8_nowait(col + TC_NH + u * 8, lo[u]);
       }
       tmem_wait_ld();
+      const float4* rh = rc + h * TC_NH + cg * 24;
 #pragma unroll
-      for (int u = 0; u < 3; ++u) {
-        if ((uint32_t)(96 * half + (3 * b + u) * 16) >= NP) continue;
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const int lr = (3 * b + u) * 16 + i;  // row within the half
-          const uint32_t row = (uint32_t)(96 * half + lr);
-          if (row < kp.rows) {
-            const RowConst rw = rc[row];
-            const float x = __uint_as_float(r3[u][i]) - rw.c32;
-            const float E = __fmaf_ru(rw.alpha, nx, rw.beta);
-            if (dbg_x && f < n) {  // diagnostic of the bound (cashash_projection_bounds)
-              dbg_x[f * kp.rows + row] = x;
-              dbg_e[f * kp.rows + row] = E;
-            }
-            if (fabsf(x) <= E) flags[lr >> 5] |= 1u << (lr & 31);
-            else if (x > 0.f) bits[lr >> 5] |= 1u << (lr & 31);
-          }
+      for (int i = 0; i < 24; ++i) {
+        const float4 k = rh[i];
+        const float x = fmaf(__uint_as_float(lo[i >> 3][i & 7]), 0x1p-11f, __uint_as_float(hi[i >> 3][i & 7])) - k.x;
+        const float E = __fmaf_ru(k.y, nx, k.z);
+        if (DBG && f < n && (uint32_t)(h * TC_NH + cg * 24 + i) < kp.rows) {
+          const uint64_t o = f * kp.rows + h * TC_NH + cg * 24 + i;
+          const int s = -__float_as_int(rcg[h * TC_NH + cg * 24 + i].pad);
+          dbg_x[o] = ldexpf(x, s);
+          dbg_e[o] = ldexpf(E, s);
         }
+        pos = __funnelshift_l(__float_as_uint(x), pos, 1);  // (x = 0 is under the bound)
+        out = __funnelshift_l(__float_as_uint(E - fabsf(x)), out, 1);
       }
+      // rows under the bound, and beyond the last row nothing
+      const int left = (int)kp.rows - (h * TC_NH + cg * 24);
+      const uint32_t live = left >= 24 ? 0xFFFFFFu : left <= 0 ? 0u : (1u << left) - 1u;
+      const uint32_t fl = (__brev(~out) >> 8) & live;
+      s_bits[b][4 * h + cg][r] = (__brev(~pos) >> 8) & live & ~fl;
+      if (fl) {  // (rare)
+        const int at = h * TC_NH + cg * 24;
+        atomicOr(&s_flag[b][at >> 5][r], fl << (at & 31));
+        if ((at & 31) > 8) atomicOr(&s_flag[b][(at >> 5) + 1][r], fl >> (32 - (at & 31)));
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      failed = __syncthreads_or(!waited);  // this half is read, and the next tile's operand written
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      if (failed) break;
+      if (tid == 0 && next < ntiles) issue(h, b ^ 1u);
     }
-    if (half == 1) {
+    if (failed) {  // never expected: record it, wait once more for all MMAs in flight, stop
+      if (tid == 0) {
+        atomicOr(status, DST_INDEX);
+        mbar_wait(smem_u32(&s_mbar[0]), phase);
+        if (next < ntiles) mbar_wait(smem_u32(&s_mbar[0]), phase ^ 1u);
+        if (halves == 2) mbar_wait(smem_u32(&s_mbar[1]), phase);
+      }
+      break;
+    }
+    // 128 threads write the tile's features; their words are not touched again before two more barriers
+    if (tid < TC_M && f < n) {
+      uint32_t w[6], fl[6];
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        s_hi[grp][k][r] = bits[k];
-        s_hi[grp][3 + k][r] = flags[k];
+      for (int h = 0; h < 2; ++h) {
+        const uint32_t a0 = s_bits[b][4 * h][r], a1 = h < halves ? s_bits[b][4 * h + 1][r] : 0u,
+                       a2 = h < halves ? s_bits[b][4 * h + 2][r] : 0u, a3 = h < halves ? s_bits[b][4 * h + 3][r] : 0u;
+        w[3 * h] = (h < halves ? a0 : 0u) | a1 << 24;
+        w[3 * h + 1] = a1 >> 8 | a2 << 16;
+        w[3 * h + 2] = a2 >> 16 | a3 << 8;
       }
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    group_sync(bar_id);
-    if (half == 0 && f < n) {
-      const uint32_t b6[6] = {bits[0], bits[1], bits[2], s_hi[grp][0][r], s_hi[grp][1][r], s_hi[grp][2][r]};
-      const uint32_t f6[6] = {flags[0], flags[1], flags[2], s_hi[grp][3][r], s_hi[grp][4][r], s_hi[grp][5][r]};
-      write_feature(f, b6, f6, sq, kp, codes, buckets, sqnorm, flagmask, flaglist, nflag_feat);
+#pragma unroll
+      for (int k = 0; k < 6; ++k) {
+        fl[k] = s_flag[b][k][r];
+        if (fl[k]) s_flag[b][k][r] = 0u;
+      }
+      write_feature(f, w, fl, kp, codes, buckets, flagmask, flaglist, nflag_feat);
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -245,29 +251,34 @@ __global__ void __launch_bounds__(PT_THREADS, 1) k_project_bf16(const uint8_t* _
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tmem), "r"(TC_TMEM_COLS) : "memory");
 }
 
-cudaError_t launch_project_bf16(const uint8_t* desc, uint64_t n, const void* Rbf, uint32_t NP, const RowConst* rc,
-                                const KParams& kp, uint32_t* codes, uint8_t* buckets, uint32_t* sqnorm,
-                                uint32_t* flagmask, uint32_t* flaglist, unsigned long long* nflag_feat,
-                                uint32_t* status, cudaStream_t s, float* dbg_x, float* dbg_e) {
+cudaError_t launch_project(const uint8_t* desc, uint64_t n, const void* Rs, uint32_t NP, const RowConst* rc,
+                           const KParams& kp, uint32_t* codes, uint8_t* buckets, uint32_t* sqnorm, uint32_t* flagmask,
+                           uint32_t* flaglist, unsigned long long* nflag_feat, uint32_t* status, cudaStream_t s,
+                           float* dbg_x, float* dbg_e) {
   if (n == 0) return cudaSuccess;
   if (NP % 16 || NP < 16 || NP > PT_ROWS_TC) return cudaErrorInvalidValue;
-  const size_t smem = 2 * (size_t)TC_M * TC_K * 2 + 2 * (size_t)NP * TC_K * 2;
+  const size_t smem = 2 * (size_t)TC_M * TC_K * 2 + 3 * (size_t)NP * TC_K * 2;
   static int attr_dev = -1;
   int dev = 0, nsm = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (attr_dev != dev) {
-    e = cudaFuncSetAttribute(k_project_bf16, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(2 * TC_M * TC_K * 2 + 2 * PT_ROWS_TC * TC_K * 2));
+    const int most = 2 * TC_M * TC_K * 2 + 3 * PT_ROWS_TC * TC_K * 2;
+    e = cudaFuncSetAttribute(k_project<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_project<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     if (e != cudaSuccess) return e;
     attr_dev = dev;
   }
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  const uint64_t ntiles = (n + TC_M - 1) / TC_M, pairs = (ntiles + 1) / 2;  // two tiles in flight per CTA
-  const int grid = (int)(pairs < (uint64_t)nsm ? pairs : (uint64_t)nsm);
-  k_project_bf16<<<grid, PT_THREADS, smem, s>>>(desc, n, reinterpret_cast<const uint4*>(Rbf), NP, rc, kp, codes,
-                                                buckets, sqnorm, flagmask, flaglist, nflag_feat, status, dbg_x,
-                                                dbg_e);
+  const uint64_t ntiles = (n + TC_M - 1) / TC_M;
+  const int grid = (int)(ntiles < (uint64_t)nsm ? ntiles : (uint64_t)nsm);
+  const uint4* R4 = reinterpret_cast<const uint4*>(Rs);
+  if (dbg_x)
+    k_project<true><<<grid, PT_THREADS, smem, s>>>(desc, n, R4, NP, rc, kp, codes, buckets, sqnorm, flagmask, flaglist,
+                                                   nflag_feat, status, dbg_x, dbg_e);
+  else
+    k_project<false><<<grid, PT_THREADS, smem, s>>>(desc, n, R4, NP, rc, kp, codes, buckets, sqnorm, flagmask,
+                                                    flaglist, nflag_feat, status, dbg_x, dbg_e);
   return cudaGetLastError();
 }
 

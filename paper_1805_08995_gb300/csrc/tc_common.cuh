@@ -1,4 +1,4 @@
-// tcgen05 building blocks shared by the tensor-core kernels (the BF16
+// tcgen05 building blocks shared by the tensor-core kernels (the
 // projection and the FP8 bucket join): shared-memory matrix descriptors, the
 // MMA and its commit to an mbarrier, a bounded mbarrier wait and tensor-memory
 // loads.  All operands use the canonical K-major layout without swizzle:
@@ -26,10 +26,10 @@ __device__ __forceinline__ uint64_t tc_desc(uint32_t saddr, uint32_t lbo, uint32
   return d;
 }
 
-// Instruction descriptor of tcgen05.mma kind::f16: D = F32, A = B = BF16,
+// Instruction descriptor of tcgen05.mma kind::f16: D = F32, A = B = F16,
 // both K-major, N >> 3 at bit 17, M >> 4 at bit 24.
-__host__ __device__ constexpr uint32_t tc_idesc(uint32_t M, uint32_t N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((N >> 3) << 17) | ((M >> 4) << 24);
+__host__ __device__ constexpr uint32_t tc_idesc_f16(uint32_t M, uint32_t N) {
+  return (1u << 4) | ((N >> 3) << 17) | ((M >> 4) << 24);
 }
 
 __device__ __forceinline__ void tc_mma(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
