@@ -366,15 +366,13 @@ int build_codes_impl(cashash_ctx* c, const cashash_set* s, const double* mean_ho
       }
       {
         StageTimer tm(c, CASHASH_STAGE_TABLES, st, capturing);
-        CK(launch_build_tables(s->buckets, c->d_chunk_feat0, c->d_chunk_len, (uint32_t)n_chunks, c->p.n_tables,
-                               s->tables, st));
-        CK(launch_build_join(s->buckets, s->codes, c->d_img_f0, c->d_img_n, c->d_img_join, s->n_images,
-                             c->p.n_tables, n_max, s->tables, st));
+        CK(launch_build_tables(s->buckets, s->codes, c->d_img_f0, c->d_img_n, c->d_img_join, s->n_images, n_max,
+                               c->d_chunk_feat0, c->d_chunk_len, (uint32_t)n_chunks, c->p.n_tables, s->tables, st));
       }
     }
     return CASHASH_OK;
   };
-  c->n_launches += (!mean_host && !sums_ready && n ? 1 : 0) + 1 + (n ? 4 : 0);
+  c->n_launches += (!mean_host && !sums_ready && n ? 1 : 0) + 1 + (n ? (tables_one_launch(n_max) ? 3 : 4) : 0);
   // A repeated build of the same set (same buffers, layout and scratch, the centre computed here)
   // replays one captured graph: the stages are a dozen short launches whose gaps would otherwise
   // show on small sets.

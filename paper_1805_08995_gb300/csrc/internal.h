@@ -259,11 +259,12 @@ cudaError_t launch_fix_fp64(const uint8_t* desc, const double* mu, const double*
                             const uint32_t* flagmask, const uint32_t* flaglist,
                             const unsigned long long* nflag_feat, uint64_t max_feat, uint32_t* codes,
                             uint8_t* buckets, unsigned long long* n_reeval, cudaStream_t s);
-cudaError_t launch_build_tables(const uint8_t* buckets, const uint64_t* chunk_feat0, const uint32_t* chunk_len,
-                                uint32_t n_chunks, uint32_t n_tables, uint8_t* tables, cudaStream_t s);
-cudaError_t launch_build_join(const uint8_t* buckets, const uint32_t* codes, const uint64_t* img_f0,
-                              const uint32_t* img_n, const uint64_t* img_join, uint32_t n_images, uint32_t n_tables,
-                              uint32_t n_max, uint8_t* join, cudaStream_t s);
+// All lookup tables of a set (tables.cu); one launch when tables_one_launch, else two.
+cudaError_t launch_build_tables(const uint8_t* buckets, const uint32_t* codes, const uint64_t* img_f0,
+                                const uint32_t* img_n, const uint64_t* img_join, uint32_t n_images, uint32_t n_max,
+                                const uint64_t* chunk_f0, const uint32_t* chunk_len, uint32_t n_chunks,
+                                uint32_t n_tables, uint8_t* tables, cudaStream_t s);
+bool tables_one_launch(uint32_t n_max);
 
 struct MatchArgs {
   const uint8_t* desc;
