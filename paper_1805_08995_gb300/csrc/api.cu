@@ -554,8 +554,8 @@ int cashash_create(cashash_ctx** out, const cashash_params* p, const double* R_h
   if (st == CASHASH_OK) st = cuda_err(cudaMemcpy(c->d_R, R_host, sizeof(double) * rows * DIM, cudaMemcpyHostToDevice));
   if (st == CASHASH_OK) st = cuda_err(cudaMemcpy(c->d_nrmR, nrm.data(), sizeof(double) * rows, cudaMemcpyHostToDevice));
   if (st == CASHASH_OK) {
-    // the three f16 terms of the scaled rows (project_tc.cu), each laid out as K-major core matrices: (row group,
-    // k group) at ((r8 * 16 + k8) * 64) elements
+    // the three f16 terms of the scaled rows (project_tc.cu), per half of up to 96 rows, each laid out as K-major core
+    // matrices: (row group, k group) at ((r8 * 16 + k8) * 64) elements
     const uint32_t NP = (rows + 15) / 16 * 16;
     c->np_tc = NP;
     std::vector<uint16_t> hb((size_t)3 * NP * DIM, 0);
@@ -573,7 +573,8 @@ int cashash_create(cashash_ctx** out, const cashash_params* p, const double* R_h
       for (int j = 0; j < DIM; ++j) {
         const double r = R_host[(size_t)b * DIM + j] * scale, hi = std::rint(r), m = (r - hi) * 2048.0;
         const double mid = std::rint(m), lo = std::rint((m - mid) * 2048.0);
-        const size_t off = ((size_t)(b >> 3) * 16 + (j >> 3)) * 64 + (b & 7) * 8 + (j & 7), part = (size_t)NP * DIM;
+        const size_t part = (size_t)(b >= 96 ? NP - 96 : std::min(NP, 96u)) * DIM, rb = b % 96;
+        const size_t off = (b / 96) * (3ull * 96 * DIM) + ((rb >> 3) * 16 + (j >> 3)) * 64 + (rb & 7) * 8 + (j & 7);
         hb[off] = f16_of_int((int)hi, 0);
         hb[part + off] = f16_of_int((int)mid, 0);
         hb[2 * part + off] = f16_of_int((int)lo, -11);

@@ -24,15 +24,16 @@
 // contiguous bytes; core matrix (r8, k8) sits at (r8 * 16 + k8) * 128 bytes, so the leading-dimension offset (next
 // core matrix along K) is 128 B and the stride offset (next 8 rows) is 2 KB.
 //
-// One CTA of 512 threads per SM, persistent over tiles of 128 features, two operand buffers.  The rows of R are
-// taken in two halves of up to 96 (one if all fit), each with its own two accumulators and mbarrier: while all warps
-// read one half back (feature row r is TMEM lane r; the four warps that may access a lane take 24 rows each), the
-// tensor cores work on the other.  773,191 features, 176 rows: 159 us (bf16 form 190); 321,454: 73 us (FP32 form 450).
-// Bound by the two barriers of a tile and by shared memory, which an MMA of 96 columns reads for 56 clocks where the
-// arithmetic takes 24 (issue 41 %, tensor pipe 28 % active).
+// One CTA per SM, persistent over tiles of 128 features, two operand buffers.  The rows of R are taken in two halves
+// of up to 96 (one if all fit), each with its own two accumulators and mbarrier: while 16 warps read one half back
+// (feature row r is TMEM lane r; the four warps that may access a lane take 24 rows each), the tensor cores work on
+// the other.  hi and mid are multiplied side by side (N = 192), which reads the features from shared memory once for
+// both.  A 17th warp issues the MMAs, so the others only announce that they have read a half (bar.arrive) and go on.
+// 773,191 features, 176 rows: 139 us (with all warps at a barrier per half and N = 96: 159; bf16 form 190); 321,454:
+// 63 us (73; FP32 form 450).  Bound by issue and the latency of the read-back (issue 46 %, tensor pipe 32 % active).
 //
-// Every wait on an MMA mbarrier is bounded; on timeout the CTA records an error, waits (bounded) for what it still
-// has in flight, stops and releases its tensor memory.
+// Every wait on an MMA mbarrier is bounded; on timeout the CTA stops issuing and waiting, still passes its barriers
+// to the end, records an error, waits (bounded) for what it has in flight and releases its tensor memory.
 #include "tc_common.cuh"
 
 namespace chx {
@@ -41,7 +42,16 @@ constexpr int TC_M = 128;
 constexpr int TC_K = 128;
 constexpr int TC_NH = 96;                // rows of R per half
 constexpr uint32_t TC_TMEM_COLS = 512;   // 2 halves x 2 accumulators x 96 columns
-constexpr int PT_THREADS = 512;
+constexpr int PT_WORK = 512;              // 16 warps convert, read back and write
+constexpr int PT_THREADS = PT_WORK + 32;  // and one issues the MMAs
+
+// Named barriers 1 and 2, one per half: "the half is read back (and the next tile's operand written)".
+__device__ __forceinline__ void half_arrive(int h) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(1 + h), "n"(PT_THREADS) : "memory");
+}
+__device__ __forceinline__ void half_sync(int h) {
+  asm volatile("bar.sync %0, %1;" ::"r"(1 + h), "n"(PT_THREADS) : "memory");
+}
 
 // Two bytes of w (half 0: bytes 0, 1; half 1: bytes 2, 3) as f16x2, exact: 0x64bb is 1024 + bb.
 __device__ __forceinline__ uint32_t f16x2_of_bytes(uint32_t w, int half) {
@@ -72,20 +82,19 @@ __global__ void __launch_bounds__(PT_THREADS, 1) k_project(const uint8_t* __rest
                                                            float* __restrict__ dbg_x, float* __restrict__ dbg_e) {
   extern __shared__ __align__(128) uint8_t tsm[];
   __shared__ __align__(8) uint64_t s_mbar[2];
-  __shared__ uint32_t s_tmem;
+  __shared__ uint32_t s_tmem, s_fail;
   __shared__ float4 rc[PT_ROWS_TC];            // c, alpha, beta
-  __shared__ float s_nx[2][TC_M];              // [tile parity][row]: ||x||
+  __shared__ float s_nx[3][TC_M];              // [tile % 3][row]: ||x||
   __shared__ uint32_t s_bits[2][8][TC_M];      // [tile parity][24 rows of R][row]: signs
   __shared__ uint32_t s_flag[2][6][TC_M];      // [tile parity][word][row]: rows under the bound (zero in between)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int cg = warp >> 2;                                       // 24 of a half's 96 rows of R
   const uint32_t r = (uint32_t)((warp & 3) * 32 + lane);          // feature row in the tile = TMEM lane
   uint8_t* As = tsm;                                              // 2 x 32 KB
-  uint8_t* Bs = tsm + 2 * (TC_M * TC_K * 2);                      // hi, mid, lo: NP x 256 B each
-  const uint32_t bbytes = NP * TC_K * 2;
+  uint8_t* Bs = tsm + 2 * (TC_M * TC_K * 2);                      // per half its rows of hi, mid and lo, 256 B each
   const int halves = NP > TC_NH ? 2 : 1;
 
-  for (uint32_t i = tid; i < 3 * bbytes / 16; i += PT_THREADS) reinterpret_cast<uint4*>(Bs)[i] = __ldg(Rs + i);
+  for (uint32_t i = tid; i < NP * (3 * TC_K * 2 / 16); i += PT_THREADS) reinterpret_cast<uint4*>(Bs)[i] = __ldg(Rs + i);
   for (int i = tid; i < PT_ROWS_TC; i += PT_THREADS) {
     RowConst z{};
     if ((uint32_t)i < kp.rows) z = rcg[i];
@@ -93,6 +102,7 @@ __global__ void __launch_bounds__(PT_THREADS, 1) k_project(const uint8_t* __rest
   }
   for (int i = tid; i < 2 * 6 * TC_M; i += PT_THREADS) (&s_flag[0][0][0])[i] = 0u;
   if (tid == 0) {
+    s_fail = 0u;
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_mbar[0])) : "memory");
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_mbar[1])) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -117,8 +127,9 @@ __global__ void __launch_bounds__(PT_THREADS, 1) k_project(const uint8_t* __rest
       v[1] = __ldg(src + 1);
     }
   };
-  // the loaded bytes -> f16 operand rows of buffer b, the norms; sqnorm is written here
-  auto convert = [&](uint64_t t, uint32_t b) {
+  // the loaded bytes -> f16 operand rows, the norms; sqnorm is written here
+  auto convert = [&](uint64_t t, uint32_t k) {  // t: the CTA's k-th tile
+    const uint32_t b = k & 1u;
     uint8_t* dst = As + b * (TC_M * TC_K * 2) + (lrow >> 3) * 2048 + (4 * part) * 128 + (lrow & 7) * 16;
     uint32_t sq = 0;
 #pragma unroll
@@ -135,113 +146,128 @@ __global__ void __launch_bounds__(PT_THREADS, 1) k_project(const uint8_t* __rest
     sq += __shfl_xor_sync(0xFFFFFFFFu, sq, 8);
     sq += __shfl_xor_sync(0xFFFFFFFFu, sq, 16);
     if (part == 0) {
-      s_nx[b][lrow] = __fsqrt_ru((float)sq);
+      s_nx[k % 3u][lrow] = __fsqrt_ru((float)sq);
       if (t * TC_M + lrow < n) sqnorm[t * TC_M + lrow] = sq;
     }
   };
-  // the MMAs of half h of the tile in buffer b (one thread)
+  // the MMAs of half h of the tile in buffer b (one thread): hi and mid side by side, then lo onto mid's columns
   auto issue = [&](int h, uint32_t b) {
-    const uint32_t rows = h ? NP - TC_NH : min(NP, (uint32_t)TC_NH), idesc = tc_idesc_f16(TC_M, rows);
-    const uint32_t a0 = smem_u32(As) + b * (TC_M * TC_K * 2), b0 = smem_u32(Bs) + (uint32_t)h * (TC_NH / 8) * 2048u;
+    const uint32_t rows = h ? NP - TC_NH : min(NP, (uint32_t)TC_NH);
+    const uint32_t a0 = smem_u32(As) + b * (TC_M * TC_K * 2), b0 = smem_u32(Bs) + (uint32_t)h * (3 * TC_NH * TC_K * 2);
     const uint32_t acc = s_tmem + (uint32_t)h * (2 * TC_NH);
 #pragma unroll
-    for (int p = 0; p < 3; ++p)
+    for (int kk = 0; kk < TC_K / 16; ++kk)
+      tc_mma(acc, tc_desc(a0 + kk * 256, 128, 2048), tc_desc(b0 + kk * 256, 128, 2048), tc_idesc_f16(TC_M, 2 * rows),
+             kk ? 1u : 0u);
 #pragma unroll
-      for (int kk = 0; kk < TC_K / 16; ++kk)
-        tc_mma(acc + (p ? TC_NH : 0), tc_desc(a0 + kk * 256, 128, 2048), tc_desc(b0 + p * bbytes + kk * 256, 128, 2048),
-               idesc, (p == 2 || kk) ? 1u : 0u);
+    for (int kk = 0; kk < TC_K / 16; ++kk)
+      tc_mma(acc + rows, tc_desc(a0 + kk * 256, 128, 2048), tc_desc(b0 + rows * (2 * TC_K * 2) + kk * 256, 128, 2048),
+             tc_idesc_f16(TC_M, rows), 1u);
     tc_commit(smem_u32(&s_mbar[h]));
   };
+  volatile uint32_t* fail = &s_fail;
 
   uint64_t tile = blockIdx.x;
-  load_tile(tile);
-  convert(tile, 0);
-  load_tile(tile + gridDim.x);
+  if (tid < PT_WORK) {
+    load_tile(tile);
+    convert(tile, 0);
+    load_tile(tile + gridDim.x);
+  }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (tid == 0)
-    for (int h = 0; h < halves; ++h) issue(h, 0);
-  const uint32_t lane_base = s_tmem + ((uint32_t)((warp & 3) * 32) << 16);
-  uint32_t phase = 0, b = 0;
-  for (; tile < ntiles; tile += gridDim.x, b ^= 1u, phase ^= 1u) {
-    const uint64_t f = tile * TC_M + r, next = tile + gridDim.x;
-    if (next < ntiles) {  // (its buffer's last MMAs were waited for in the previous round)
-      convert(next, b ^ 1u);
-      load_tile(next + gridDim.x);
-    }
-    const float nx = s_nx[b][r];
-    bool failed = false;
-    for (int h = 0; h < halves; ++h) {
-      const bool waited = mbar_wait(smem_u32(&s_mbar[h]), phase);
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t col = lane_base + (uint32_t)(h * 2 * TC_NH + cg * 24);
-      uint32_t hi[3][8], lo[3][8], pos = 0, out = 0;  // bit 23 - i: row i's sign, and whether it is outside the bound
-#pragma unroll
-      for (int u = 0; u < 3; ++u) {
-        tmem_ld8_nowait(col + u * 8, hi[u]);
-        tmem_ld8_nowait(col + TC_NH + u * 8, lo[u]);
+  if (tid >= PT_WORK) {  // the issuing warp: a half's next MMAs once all have read its accumulators
+    if (lane == 0)
+      for (int h = 0; h < halves; ++h) issue(h, 0);
+    uint32_t issued = 1;  // tiles whose MMAs are issued (of half 0; of half 1 after each round)
+    for (uint32_t b = 1; tile < ntiles; tile += gridDim.x, b ^= 1u) {
+      const bool more = tile + gridDim.x < ntiles;
+      for (int h = 0; h < halves; ++h) {
+        half_sync(h);
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        if (lane == 0 && more && !*fail) issue(h, b);
       }
-      tmem_wait_ld();
-      const float4* rh = rc + h * TC_NH + cg * 24;
+      issued += more ? 1u : 0u;
+    }
+    if (lane == 0 && *fail) {  // never expected: record it; what is in flight gets another (bounded) wait
+      atomicOr(status, DST_INDEX);
+      for (uint32_t i = 0; i < 2; ++i)
+        for (int h = 0; h < halves; ++h) mbar_wait(smem_u32(&s_mbar[h]), i ^ (issued & 1u));
+    }
+  } else {
+    const uint32_t lane_base = s_tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    for (uint32_t k = 0; tile < ntiles; tile += gridDim.x, ++k) {
+      const uint32_t b = k & 1u;
+      const uint64_t f = tile * TC_M + r, next = tile + gridDim.x;
+      if (next < ntiles) {  // (this thread waited for all MMAs of that buffer in the previous round)
+        convert(next, k + 1);
+        load_tile(next + gridDim.x);
+      }
+      float nx = 0.f;
+      for (int h = 0; h < halves; ++h) {
+        if (!*fail && !mbar_wait(smem_u32(&s_mbar[h]), b)) *fail = 1u;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        if (h == 0) nx = s_nx[k % 3u][r];  // (written before the barrier that this half's MMAs waited for)
+        const uint32_t col = lane_base + (uint32_t)(h * 2 * TC_NH + cg * 24);
+        const uint32_t rows = h ? NP - TC_NH : min(NP, (uint32_t)TC_NH);
+        uint32_t hi[3][8], lo[3][8], pos = 0, out = 0;  // bit 23 - i: row i's sign, and whether it is outside the bound
 #pragma unroll
-      for (int i = 0; i < 24; ++i) {
-        const float4 k = rh[i];
-        const float x = fmaf(__uint_as_float(lo[i >> 3][i & 7]), 0x1p-11f, __uint_as_float(hi[i >> 3][i & 7])) - k.x;
-        const float E = __fmaf_ru(k.y, nx, k.z);
-        if (DBG && f < n && (uint32_t)(h * TC_NH + cg * 24 + i) < kp.rows) {
-          const uint64_t o = f * kp.rows + h * TC_NH + cg * 24 + i;
-          const int s = -__float_as_int(rcg[h * TC_NH + cg * 24 + i].pad);
-          dbg_x[o] = ldexpf(x, s);
-          dbg_e[o] = ldexpf(E, s);
+        for (int u = 0; u < 3; ++u) {
+          tmem_ld8_nowait(col + u * 8, hi[u]);
+          tmem_ld8_nowait(col + rows + u * 8, lo[u]);
         }
-        pos = __funnelshift_l(__float_as_uint(x), pos, 1);  // (x = 0 is under the bound)
-        out = __funnelshift_l(__float_as_uint(E - fabsf(x)), out, 1);
-      }
-      // rows under the bound, and beyond the last row nothing
-      const int left = (int)kp.rows - (h * TC_NH + cg * 24);
-      const uint32_t live = left >= 24 ? 0xFFFFFFu : left <= 0 ? 0u : (1u << left) - 1u;
-      const uint32_t fl = (__brev(~out) >> 8) & live;
-      s_bits[b][4 * h + cg][r] = (__brev(~pos) >> 8) & live & ~fl;
-      if (fl) {  // (rare)
-        const int at = h * TC_NH + cg * 24;
-        atomicOr(&s_flag[b][at >> 5][r], fl << (at & 31));
-        if ((at & 31) > 8) atomicOr(&s_flag[b][(at >> 5) + 1][r], fl >> (32 - (at & 31)));
-      }
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      failed = __syncthreads_or(!waited);  // this half is read, and the next tile's operand written
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      if (failed) break;
-      if (tid == 0 && next < ntiles) issue(h, b ^ 1u);
-    }
-    if (failed) {  // never expected: record it, wait once more for all MMAs in flight, stop
-      if (tid == 0) {
-        atomicOr(status, DST_INDEX);
-        mbar_wait(smem_u32(&s_mbar[0]), phase);
-        if (next < ntiles) mbar_wait(smem_u32(&s_mbar[0]), phase ^ 1u);
-        if (halves == 2) mbar_wait(smem_u32(&s_mbar[1]), phase);
-      }
-      break;
-    }
-    // 128 threads write the tile's features; their words are not touched again before two more barriers
-    if (tid < TC_M && f < n) {
-      uint32_t w[6], fl[6];
+        tmem_wait_ld();
+        const float4* rh = rc + h * TC_NH + cg * 24;
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const uint32_t a0 = s_bits[b][4 * h][r], a1 = h < halves ? s_bits[b][4 * h + 1][r] : 0u,
-                       a2 = h < halves ? s_bits[b][4 * h + 2][r] : 0u, a3 = h < halves ? s_bits[b][4 * h + 3][r] : 0u;
-        w[3 * h] = (h < halves ? a0 : 0u) | a1 << 24;
-        w[3 * h + 1] = a1 >> 8 | a2 << 16;
-        w[3 * h + 2] = a2 >> 16 | a3 << 8;
+        for (int i = 0; i < 24; ++i) {
+          const float4 c = rh[i];
+          const float x = fmaf(__uint_as_float(lo[i >> 3][i & 7]), 0x1p-11f, __uint_as_float(hi[i >> 3][i & 7])) - c.x;
+          const float E = __fmaf_ru(c.y, nx, c.z);
+          if (DBG && f < n && (uint32_t)(h * TC_NH + cg * 24 + i) < kp.rows) {
+            const uint64_t o = f * kp.rows + h * TC_NH + cg * 24 + i;
+            const int s = -__float_as_int(rcg[h * TC_NH + cg * 24 + i].pad);
+            dbg_x[o] = ldexpf(x, s);
+            dbg_e[o] = ldexpf(E, s);
+          }
+          pos = __funnelshift_l(__float_as_uint(x), pos, 1);  // (x = 0 is under the bound)
+          out = __funnelshift_l(__float_as_uint(E - fabsf(x)), out, 1);
+        }
+        // rows under the bound, and beyond the last row nothing
+        const int left = (int)kp.rows - (h * TC_NH + cg * 24);
+        const uint32_t live = left >= 24 ? 0xFFFFFFu : left <= 0 ? 0u : (1u << left) - 1u;
+        const uint32_t fl = (__brev(~out) >> 8) & live;
+        s_bits[b][4 * h + cg][r] = (__brev(~pos) >> 8) & live & ~fl;
+        if (fl) {  // (rare)
+          const int at = h * TC_NH + cg * 24;
+          atomicOr(&s_flag[b][at >> 5][r], fl << (at & 31));
+          if ((at & 31) > 8) atomicOr(&s_flag[b][(at >> 5) + 1][r], fl >> (32 - (at & 31)));
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __threadfence_block();
+        if (h + 1 == halves && cg == 0) half_sync(h);  // the warps that write wait for all signs of the tile
+        else half_arrive(h);
       }
+      // (the words of a parity are written again only after MMAs that wait for these warps' next arrival)
+      if (cg == 0 && f < n && !*fail) {
+        uint32_t w[6], fl[6];
 #pragma unroll
-      for (int k = 0; k < 6; ++k) {
-        fl[k] = s_flag[b][k][r];
-        if (fl[k]) s_flag[b][k][r] = 0u;
+        for (int h = 0; h < 2; ++h) {
+          uint32_t a[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) a[i] = h < halves ? s_bits[b][4 * h + i][r] : 0u;
+          w[3 * h] = a[0] | a[1] << 24;
+          w[3 * h + 1] = a[1] >> 8 | a[2] << 16;
+          w[3 * h + 2] = a[2] >> 16 | a[3] << 8;
+        }
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+          fl[i] = s_flag[b][i][r];
+          if (fl[i]) s_flag[b][i][r] = 0u;
+        }
+        write_feature(f, w, fl, kp, codes, buckets, flagmask, flaglist, nflag_feat);
       }
-      write_feature(f, w, fl, kp, codes, buckets, flagmask, flaglist, nflag_feat);
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
