@@ -28,12 +28,15 @@
 // of up to 96 (one if all fit), each with its own two accumulators and mbarrier: while 16 warps read one half back
 // (feature row r is TMEM lane r; the four warps that may access a lane take 24 rows each), the tensor cores work on
 // the other.  hi and mid are multiplied side by side (N = 192), which reads the features from shared memory once for
-// both.  A 17th warp issues the MMAs, so the others only announce that they have read a half (bar.arrive) and go on.
+// both.  A 17th warp issues the MMAs, so the others only announce that they have read a half (an arrival on the half's
+// second mbarrier) and go on.
 // 773,191 features, 176 rows: 139 us (with all warps at a barrier per half and N = 96: 159; bf16 form 190); 321,454:
 // 63 us (73; FP32 form 450).  Bound by issue and the latency of the read-back (issue 46 %, tensor pipe 32 % active).
 //
-// Every wait on an MMA mbarrier is bounded; on timeout the CTA stops issuing and waiting, still passes its barriers
-// to the end, records an error, waits (bounded) for what it has in flight and releases its tensor memory.
+// Every wait between the first tile and the last is a bounded one on an mbarrier: for a half's MMAs, for all warps to
+// have read a half, for the signs of a tile.  A warp whose wait times out records an error and leaves its loop; those
+// that depend on it leave at a time-out of their own.  The issuing warp then waits (bounded) for what is in flight, all
+// warps meet at the last barrier, and the tensor memory is released.
 #include "tc_common.cuh"
 
 namespace chx {
@@ -45,12 +48,10 @@ constexpr uint32_t TC_TMEM_COLS = 512;   // 2 halves x 2 accumulators x 96 colum
 constexpr int PT_WORK = 512;              // 16 warps convert, read back and write
 constexpr int PT_THREADS = PT_WORK + 32;  // and one issues the MMAs
 
-// Named barriers 1 and 2, one per half: "the half is read back (and the next tile's operand written)".
-__device__ __forceinline__ void half_arrive(int h) {
-  asm volatile("bar.arrive %0, %1;" ::"r"(1 + h), "n"(PT_THREADS) : "memory");
-}
-__device__ __forceinline__ void half_sync(int h) {
-  asm volatile("bar.sync %0, %1;" ::"r"(1 + h), "n"(PT_THREADS) : "memory");
+// One arrival on an mbarrier for the whole warp, after what its lanes have read and written.
+__device__ __forceinline__ void warp_arrive(uint32_t mbar, int lane) {
+  __syncwarp();
+  if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mbar) : "memory");
 }
 
 // Two bytes of w (half 0: bytes 0, 1; half 1: bytes 2, 3) as f16x2, exact: 0x64bb is 1024 + bb.
@@ -81,8 +82,9 @@ __global__ void __launch_bounds__(PT_THREADS, 1) k_project(const uint8_t* __rest
                                                            uint32_t* __restrict__ status,
                                                            float* __restrict__ dbg_x, float* __restrict__ dbg_e) {
   extern __shared__ __align__(128) uint8_t tsm[];
-  __shared__ __align__(8) uint64_t s_mbar[2];
-  __shared__ uint32_t s_tmem, s_fail;
+  __shared__ __align__(8) uint64_t s_mbar[2];  // per half: its MMAs are done
+  __shared__ __align__(8) uint64_t s_read[2];  // per half: every warp has read it (and written the next tile's operand)
+  __shared__ uint32_t s_tmem;
   __shared__ float4 rc[PT_ROWS_TC];            // c, alpha, beta
   __shared__ float s_nx[3][TC_M];              // [tile % 3][row]: ||x||
   __shared__ uint32_t s_bits[2][8][TC_M];      // [tile parity][24 rows of R][row]: signs
@@ -102,9 +104,10 @@ __global__ void __launch_bounds__(PT_THREADS, 1) k_project(const uint8_t* __rest
   }
   for (int i = tid; i < 2 * 6 * TC_M; i += PT_THREADS) (&s_flag[0][0][0])[i] = 0u;
   if (tid == 0) {
-    s_fail = 0u;
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_mbar[0])) : "memory");
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_mbar[1])) : "memory");
+    for (int h = 0; h < 2; ++h) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_mbar[h])) : "memory");
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&s_read[h])), "n"(PT_WORK / 32) : "memory");
+    }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
@@ -165,7 +168,12 @@ __global__ void __launch_bounds__(PT_THREADS, 1) k_project(const uint8_t* __rest
              tc_idesc_f16(TC_M, rows), 1u);
     tc_commit(smem_u32(&s_mbar[h]));
   };
-  volatile uint32_t* fail = &s_fail;
+  // the whole warp waits for a phase; false: the wait timed out
+  auto wait_all = [&](uint64_t* mbar, uint32_t parity) {
+    const bool ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(mbar), parity));
+    if (!ok && lane == 0) atomicOr(status, DST_INDEX);  // never expected
+    return ok;
+  };
 
   uint64_t tile = blockIdx.x;
   if (tid < PT_WORK) {
@@ -178,26 +186,25 @@ __global__ void __launch_bounds__(PT_THREADS, 1) k_project(const uint8_t* __rest
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (tid >= PT_WORK) {  // the issuing warp: a half's next MMAs once all have read its accumulators
+    uint32_t last = 0;  // bit h: parity of the phase that half h's latest MMAs complete
     if (lane == 0)
       for (int h = 0; h < halves; ++h) issue(h, 0);
-    uint32_t issued = 1;  // tiles whose MMAs are issued (of half 0; of half 1 after each round)
-    for (uint32_t b = 1; tile < ntiles; tile += gridDim.x, b ^= 1u) {
-      const bool more = tile + gridDim.x < ntiles;
+    bool ok = true;
+    for (uint32_t k = 0; ok && tile + gridDim.x < ntiles; tile += gridDim.x, ++k) {
       for (int h = 0; h < halves; ++h) {
-        half_sync(h);
+        ok = wait_all(&s_read[h], k & 1u);
+        if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        if (lane == 0 && more && !*fail) issue(h, b);
+        if (lane == 0) issue(h, (k + 1) & 1u);
+        last ^= 1u << h;
       }
-      issued += more ? 1u : 0u;
     }
-    if (lane == 0 && *fail) {  // never expected: record it; what is in flight gets another (bounded) wait
-      atomicOr(status, DST_INDEX);
-      for (uint32_t i = 0; i < 2; ++i)
-        for (int h = 0; h < halves; ++h) mbar_wait(smem_u32(&s_mbar[h]), i ^ (issued & 1u));
-    }
+    // whatever ended the loop: no operand, accumulator or mbarrier goes before the last MMAs are done
+    for (int h = 0; h < halves; ++h) wait_all(&s_mbar[h], last >> h & 1u);
   } else {
     const uint32_t lane_base = s_tmem + ((uint32_t)((warp & 3) * 32) << 16);
-    for (uint32_t k = 0; tile < ntiles; tile += gridDim.x, ++k) {
+    bool ok = true;
+    for (uint32_t k = 0; ok && tile < ntiles; tile += gridDim.x, ++k) {
       const uint32_t b = k & 1u;
       const uint64_t f = tile * TC_M + r, next = tile + gridDim.x;
       if (next < ntiles) {  // (this thread waited for all MMAs of that buffer in the previous round)
@@ -206,7 +213,8 @@ __global__ void __launch_bounds__(PT_THREADS, 1) k_project(const uint8_t* __rest
       }
       float nx = 0.f;
       for (int h = 0; h < halves; ++h) {
-        if (!*fail && !mbar_wait(smem_u32(&s_mbar[h]), b)) *fail = 1u;
+        ok = wait_all(&s_mbar[h], b);
+        if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if (h == 0) nx = s_nx[k % 3u][r];  // (written before the barrier that this half's MMAs waited for)
         const uint32_t col = lane_base + (uint32_t)(h * 2 * TC_NH + cg * 24);
@@ -245,12 +253,12 @@ __global__ void __launch_bounds__(PT_THREADS, 1) k_project(const uint8_t* __rest
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __threadfence_block();
-        if (h + 1 == halves && cg == 0) half_sync(h);  // the warps that write wait for all signs of the tile
-        else half_arrive(h);
+        warp_arrive(smem_u32(&s_read[h]), lane);
       }
+      if (!ok) break;
+      if (cg == 0 && !wait_all(&s_read[halves - 1], b)) break;  // the warps that write wait for all signs of the tile
       // (the words of a parity are written again only after MMAs that wait for these warps' next arrival)
-      if (cg == 0 && f < n && !*fail) {
+      if (cg == 0 && f < n) {
         uint32_t w[6], fl[6];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
