@@ -40,8 +40,8 @@ L2_FLUSH_BYTES = 256 << 20
 # summarised in profiles/ (valid only for the kernel source it was taken on).
 PROFILED_TRAFFIC = {
     "k_join": {"sources": ["paper_1805_08995_gb300/csrc/join.cu", "paper_1805_08995_gb300/csrc/join_common.cuh"],
-               "sha256": "760d0f459ce8a365b5e559bec372a5b6e2526701eccbbd5af224cf385442736a",
-               "bytes_per_entry": (2.565599e9 + 1.097986e9) / 861951265},
+               "sha256": "543165e038126155e711ec0220c19d991005eb1c058ab392ba3fe8e786caf9f8",
+               "bytes_per_entry": (2.633339e9 + 1.099100e9) / 861951265},
 }
 
 

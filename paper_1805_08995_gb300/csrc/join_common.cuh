@@ -12,6 +12,7 @@ namespace chx {
 
 constexpr int JT = 256;  // threads of a CTA of the tcgen05 form
 
+// Insertion that drops a key equal to one already kept.
 template <int KC>
 __device__ __forceinline__ void jt_insert(uint32_t (&top)[KC], uint32_t k) {
 #pragma unroll
@@ -99,14 +100,43 @@ __device__ __forceinline__ uint32_t pair_threshold(const MatchArgs& a, uint32_t 
 // Words per query of the finalisation's keys and distances.
 __host__ __device__ constexpr int join_kp(int KC) { return (KC + 3) / 4 * 4; }
 
+// The K <= KC smallest distinct keys of a survivor list of m <= JSEG entries, ascending, then KEY_INF, to keys[KC].
+// Not inlined: the finalisation's own pass would pay for its registers.
+template <int KC>
+__device__ __noinline__ void jt_distinct(const uint32_t* list, uint32_t m, uint32_t K, uint32_t* keys) {
+  uint32_t top[KC];
+#pragma unroll
+  for (int s = 0; s < KC; ++s) top[s] = KEY_INF;
+#pragma unroll 1
+  for (uint32_t e0 = 0; e0 < m; e0 += 4) {
+    const uint4 x = __ldcg(reinterpret_cast<const uint4*>(list) + e0 / 4);  // (the list has JSEG entries)
+    const uint32_t kk[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (e0 + u < m && kk[u] < top[KC - 1]) jt_insert<KC>(top, kk[u]);
+  }
+#pragma unroll
+  for (int s = 0; s < KC; ++s) keys[s] = (uint32_t)s < K ? top[s] : KEY_INF;
+}
+
+// Whether a query meets most of its candidates in several tables, so that the finalisation reads its list by
+// jt_distinct at once.  us per pass over 400 pairs, 6 tables, after a pass that keeps repeats / at once: 6,000 x 6,000
+// features, 7 bits k = 10 1,524 / 1,513, k = 16 2,060 / 2,014; 6 bits 2,002 / 1,930 and 3,112 / 2,717; 4 bits, k = 10
+// 9,724 / 9,162; 1,000 x 1,000, 7 bits k = 32 1,023 / 858.  With 8 bits few queries have repeats beyond the spare entries.
+__host__ __device__ inline bool join_repeats(const KParams& kp) { return kp.n_tables > 1 && kp.bits_per_table <= 7; }
+
 // Finalisation of up to 32 queries of a pair by one warp, the lane's query q (valid: it exists) with n keys
 // counted in its survivor list: the k smallest distinct survivors (Step 3), exact squared distances of those k
 // with 4 lanes per 128-byte row (Step 4, Sec. 5.2) and Lowe's ratio test.  A query whose list overflowed, or
 // that holds fewer than k survivors while the guess may have turned a candidate away (cut), is left PENDING for
 // the exact fallback.  key_s, dist_s: 32 join_kp(KC) words each, the warp's own.
 // Bound by issue: the insertion network keeps equal keys (two independent operations per entry instead of four
-// dependent ones; repeats are dropped once at the end) and the distances take 67 instructions per four rows of
+// dependent ones; repeats are dropped once at the end, and where that loses keys, or would for most queries, the list
+// is read by jt_distinct) and the distances take 67 instructions per four rows of
 // eight queries (one exchange tree for four sums).  Per 32 queries about 3,100 warp instructions, 4,500 before.
+// Queries that lose keys to repeats are not left to the fallback: with that, 400 pairs of 1,000 x 1,000 features, 8
+// tables of 4 bits, k = 10 took 1,140 us a pass, now 570; 6,000 x 6,000 25.5 ms, now 12.2; images of near copies of
+// each descriptor, 6 tables of 8 bits, 6,000 x 6,000 3,745 us, now 1,663.
 template <int KC, bool EPI>
 __device__ __forceinline__ void finalise_warp(const MatchArgs& a, const PairInfo& P, uint32_t it, bool cut, uint32_t q,
                                               bool valid, uint32_t n, const uint32_t* list, uint32_t* key_s,
@@ -119,11 +149,11 @@ __device__ __forceinline__ void finalise_warp(const MatchArgs& a, const PairInfo
   uint32_t top[KN];
 #pragma unroll
   for (int s = 0; s < KN; ++s) top[s] = KEY_INF;
-  bool pending = false;
+  bool pending = false, again = join_repeats(kp);  // again: the keys come from jt_distinct
   if (valid) {
     pending = n > JSEG;  // survivors were dropped
     const uint4* ql = reinterpret_cast<const uint4*>(list);
-    const uint32_t m = min(n, JSEG);
+    const uint32_t m = again ? 0u : min(n, JSEG);
     // a key at or above the list's last entry when its group of eight starts cannot enter it
     for (uint32_t e0 = 0; e0 < m; e0 += 8) {
       const uint4 x0 = __ldcg(ql + e0 / 4), x1 = __ldcg(ql + e0 / 4 + 1);  // (the list has JSEG entries)
@@ -147,9 +177,26 @@ __device__ __forceinline__ void finalise_warp(const MatchArgs& a, const PairInfo
         }
         if (!seen) break;
       }
-      if (full && jt_kth<KC>(top, K) == KEY_INF) pending = true;
+      again = full && jt_kth<KC>(top, K) == KEY_INF;
     }
-    const uint32_t kth = jt_kth<KC>(top, K);
+  }
+  again = again && valid && !pending;
+  uint32_t* keys = key_s + lane * KP;
+#pragma unroll
+  for (int s = 0; s < KP; s += 4) {
+    const bool ok = valid && !pending;
+    uint4 k4;
+    k4.x = ok && (uint32_t)s < K ? top[s] : KEY_INF;
+    k4.y = ok && (uint32_t)s + 1 < K ? top[s + 1 < KN ? s + 1 : 0] : KEY_INF;
+    k4.z = ok && (uint32_t)s + 2 < K ? top[s + 2 < KN ? s + 2 : 0] : KEY_INF;
+    k4.w = ok && (uint32_t)s + 3 < K ? top[s + 3 < KN ? s + 3 : 0] : KEY_INF;
+    *reinterpret_cast<uint4*>(keys + s) = k4;
+  }
+  if (__any_sync(0xFFFFFFFFu, again)) {  // (top is not needed any more: a call here costs the others nothing)
+    if (again) jt_distinct<KC>(list, n, K, keys);
+  }
+  if (valid) {
+    const uint32_t kth = keys[K - 1];
     if (!pending && kth == KEY_INF && cut) {
       // fewer than k: exact only if no candidate was turned away by the guess
       const uint2 qbk = __ldg(reinterpret_cast<const uint2*>(a.buckets) + P.a0 + q);
@@ -160,18 +207,10 @@ __device__ __forceinline__ void finalise_warp(const MatchArgs& a, const PairInfo
         nlook += __ldg(B.off + v + 1) - __ldg(B.off + v);
       }
       pending = nlook > n;
+      if (pending)
+        for (uint32_t s = 0; s < K; ++s) keys[s] = KEY_INF;
     }
     if (!EPI && !pending && kth != KEY_INF && !a.tau_fixed) atomicAdd(s_hist + (kth >> 24), 1u);
-  }
-#pragma unroll
-  for (int s = 0; s < KP; s += 4) {
-    const bool ok = valid && !pending;
-    uint4 k4;
-    k4.x = ok && (uint32_t)s < K ? top[s] : KEY_INF;
-    k4.y = ok && (uint32_t)s + 1 < K ? top[s + 1 < KN ? s + 1 : 0] : KEY_INF;
-    k4.z = ok && (uint32_t)s + 2 < K ? top[s + 2 < KN ? s + 2 : 0] : KEY_INF;
-    k4.w = ok && (uint32_t)s + 3 < K ? top[s + 3 < KN ? s + 3 : 0] : KEY_INF;
-    *reinterpret_cast<uint4*>(key_s + lane * KP + s) = k4;
   }
   __syncwarp();
   // 4 lanes per 128-byte row (32 bytes each), 8 queries per step, four candidates' rows in flight; a missing
