@@ -209,8 +209,9 @@ __global__ void __launch_bounds__(256) k_build_join(const uint8_t* __restrict__ 
 }
 
 // Image and chunk tables in one launch while the images' shared memory leaves room for four CTAs of an SM, as many
-// as its threads do (13,653 features); else the chunks would run fewer at a time than they can.
-bool tables_one_launch(uint32_t n_max) { return sort_smem(n_max) <= 56 * 1024; }
+// as its threads do (up to 13,640 features); else the chunks would run fewer at a time than they can.  An SM has 228
+// KB, of which the system takes 1 KB for each CTA and the kernel's static arrays 32 bytes.
+bool tables_one_launch(uint32_t n_max) { return sort_smem(n_max) <= 228 * 1024 / 4 - 1024 - 32; }
 
 cudaError_t launch_build_tables(const uint8_t* buckets, const uint32_t* codes, const uint64_t* img_f0,
                                 const uint32_t* img_n, const uint64_t* img_join, uint32_t n_images, uint32_t n_max,
