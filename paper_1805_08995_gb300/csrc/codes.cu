@@ -58,7 +58,7 @@ cudaError_t launch_colsum(const uint8_t* desc, uint64_t n, unsigned long long* s
 // division).  c_b = sum_j R_bj mu_j is needed only by the approximation, so
 // its summation order is free; its error enters the bound.
 //   |v~ - v_double| <= alpha_b ||x||_2 + beta_b (project_tc.cu), all in units of 2^-s_b,
-//     alpha_b = 2^-21 max(2^s ||R_b||_2, 256),
+//     alpha_b = 2^-20 max(2^s ||R_b||_2, 256),
 //     beta_b  = 2^s (2^-23 |c_b| + 2^-40 ||R_b||_2 (||mu||_2 + 1)).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_row_consts(const unsigned long long* __restrict__ sums, uint64_t n,
@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(256) k_row_consts(const unsigned long long* __
       const int e = expo[b];
       const double nr = scalbn(nrmR[b], e);
       r.c32 = (float)scalbn(c, e);
-      r.alpha = (float)(0x1p-21 * fmax(nr, 256.0) * (1.0 + 0x1p-20));
+      r.alpha = (float)(0x1p-20 * fmax(nr, 256.0) * (1.0 + 0x1p-20));
       r.beta = (float)((0x1p-23 * fabs(scalbn(c, e)) + 0x1p-40 * nr * (nmu_s + 1.0)) * (1.0 + 0x1p-20) + 0x1p-60);
       r.pad = __int_as_float(e);
       rc[b] = r;

@@ -8,17 +8,20 @@
 // FP32 in any order.  A second one takes X mid^T, then X lo^T, and enters at 2^-11.  Error of A + 2^-11 B - c
 // against 2^s v, in units of N = max(2^s ||R_b||, 256) ||x||:
 //   * the split: |r - hi - 2^-11 (mid + lo)| <= 2^-23, so at most 2^-23 sum x <= 2^-23 sqrt(128) ||x|| < 2^-27 N;
-//   * B with a pessimistic adder (every step truncates, no guard bits): 33 * 2^-23 sum x |mid + lo| with |mid| <=
-//     1024, at 2^-11 half of 33 * 2^-23 sqrt(128) ||x||, below 2^-23.4 N for a row with one large entry (for rows
-//     of normal numbers, N = 1900 ||x||, eight times less);
+//   * B, 16 MMAs of 16 products.  How the tensor cores add is not documented; taken here: each MMA aligns its products
+//     and the accumulator to the largest of them and cuts all off below its 24th bit, and the sum as well (A stays
+//     exact under that: integers).  288 cuts of at most 2^-23 S each, S = sum x (|mid| + |lo|) <= 1024.5 sqrt(128)
+//     ||x||, at 2^-11: below 2^-20.3 N for a row with one large entry (N = 256 ||x||; for rows of normal numbers, N =
+//     1900 ||x||, seven times less);
 //   * A + 2^-11 B rounded: 2^-24 N; minus c: 2^-24 (N + |c|), and c is rounded itself: beta has 2^-23 |c|.
-// The sum is below 2^-22.2 N; the flag test takes 2^-21 N plus beta (which has the rounding of the double sequence
+// The sum is below 2^-20.1 N; the flag test takes 2^-20 N plus beta (which has the rounding of the double sequence
 // too).  |v~| under the bound goes to k_fix_fp64, so the signs equal the double definition.
 //
 // Before, the FP32 setting took CUDA-core FMA chains over 24-bit weights (bound 2^-16) and the other one a two-term
 // bf16 split (2^-15).  Against the doubles, over 60,000 features and 176 rows of normal numbers: error 1.9e-5 rms and
 // 1.7e-4 at most, where the FMA chains had 1.1e-4 and 1.5e-3 and the bf16 split 1.3e-3 and 6.6e-3; of 844,018
-// features 1,063 projections are re-evaluated, where it was 34,262 and 68,755.
+// features 2,169 projections are re-evaluated, where it was 34,262 and 68,755 (1,063 with half the bound, which a row of
+// one large entry could exceed; 773,191 features 2 us a build).
 //
 // Shared-memory operands use the canonical K-major layout without swizzle: 8-row x 16-byte core matrices of 128
 // contiguous bytes; core matrix (r8, k8) sits at (r8 * 16 + k8) * 128 bytes, so the leading-dimension offset (next
