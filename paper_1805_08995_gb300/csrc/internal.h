@@ -309,13 +309,13 @@ uint32_t join_grid(const KParams& kp, uint32_t na_max, uint32_t n_items, uint32_
 // memory; and the launch.
 uint32_t join_tc_grid(const KParams& kp, uint32_t na_max, uint32_t n_items, uint32_t ctas_per_sm);
 cudaError_t launch_join_tc(const MatchArgs& a, uint32_t grid, cudaStream_t s);
-// Matching kernel launch.  spec = 0: direct register top-k (one pair per
-// launch); spec = 1: survivor queues with a speculative threshold (batched).
-// tile: queries per CTA of the speculative form (256, or 512 when k <= 16; 0 = default).
 // One pair on its own, a warp per query (match_pair_by_warps: where that is faster than launch_match with spec = 0);
 // after: the launch before it on the stream is such a one, of another pair.
 bool match_pair_by_warps(const KParams& kp, uint32_t nA, uint32_t nB);
 cudaError_t launch_match_pair(const MatchArgs& a, uint32_t pair, const PairInfo& P, bool after, cudaStream_t s);
+// Matching kernel launch.  spec = 0: direct register top-k (one pair per
+// launch); spec = 1: survivor queues with a speculative threshold (batched).
+// tile: queries per CTA of the speculative form (256, or 512 when k <= 16; 0 = default).
 cudaError_t launch_match(const MatchArgs& a, int spec, uint32_t grid, cudaStream_t s, uint32_t tile = 0);
 // Largest useful grid (resident CTAs) for a launch over n_items items.
 uint32_t match_grid(uint32_t top_k, int spec, bool epi, uint32_t n_tables, uint32_t n_items, uint32_t tile = 0);

@@ -515,7 +515,9 @@ cudaError_t run_match(const MatchArgs* a, uint32_t grid, cudaStream_t s, uint32_
 template <int KC, int TPB>
 cudaError_t run_kc(const MatchArgs* a, int spec, bool epi, uint32_t grid, cudaStream_t s, uint32_t* occ) {
   if (spec) return epi ? run_match<KC, TPB, true, true>(a, grid, s, occ) : run_match<KC, TPB, false, true>(a, grid, s, occ);
-  return epi ? run_match<KC, TPB, true, false>(a, grid, s, occ) : run_match<KC, TPB, false, false>(a, grid, s, occ);
+  if constexpr (TPB == 256)  // (the direct form has 256 queries per CTA)
+    return epi ? run_match<KC, TPB, true, false>(a, grid, s, occ) : run_match<KC, TPB, false, false>(a, grid, s, occ);
+  return cudaErrorInvalidValue;
 }
 
 // Queries per CTA of the speculative form: 512 (k <= 16 only) or 256.
