@@ -204,13 +204,13 @@ void cashash_plan_destroy(cashash_plan* plan);
  * match_off is still complete, nothing beyond cap is written and
  * cashash_sync_status() returns EOVERFLOW.  Asynchronous on `stream`.
  * With the persistent schedule all pairs are matched by one batched kernel:
- * by default a warp per query for at most three pairs of images of up to
- * 65,535 features; else a bucket join when every query image has at most about
- * 50,000 features (at least 40,000 whatever the parameters), else a speculative
- * per-query kernel (cashash_plan_autotune may choose otherwise); the launch
- * sequence is captured once as a CUDA graph (per set of output pointers, F and
- * profiling setting) and replayed on `stream`; calls on the same plan must
- * not overlap.
+ * by default a speculative per-query kernel when a query image has more than
+ * about 50,000 features (more than 40,000 for large top_k); else a warp per
+ * query for at most three matched pairs of images of up to 65,535 features (with
+ * the mutual check every pair is matched twice); else a bucket join
+ * (cashash_plan_autotune may choose otherwise); the launch sequence is captured
+ * once as a CUDA graph (per set of output pointers, F and profiling setting) and
+ * replayed on `stream`; calls on the same plan must not overlap.
  * Errors: EINVAL, ECUDA. */
 int cashash_match_plan(cashash_ctx* ctx, cashash_plan* plan, const double* F_dev, uint64_t* match_off,
                        uint32_t* matches, uint64_t cap, cashash_stream_t stream);
@@ -220,7 +220,8 @@ int cashash_match_plan(cashash_ctx* ctx, cashash_plan* plan, const double* F_dev
  * starts.  The kernels then adapt it per pair to the k-th ranked distances
  * they observe (unless `fixed` is non-zero).  Results never depend on it: a
  * query for which the hint turns away candidates it needed is re-matched
- * exactly.  hamming >= code_bits disables the speculation.
+ * exactly.  hamming >= code_bits disables the speculation.  The warp-per-query
+ * kernel takes no threshold.
  * Errors: EINVAL, ECUDA. */
 int cashash_plan_set_threshold_hint(cashash_plan* plan, uint32_t hamming, int fixed);
 
@@ -247,8 +248,8 @@ typedef struct {
                             this configuration; -1 otherwise */
 } cashash_tuning;
 
-/* The configuration a plan matches with (chosen at creation: the join when it
- * applies, else the per-query kernel).  Errors: EINVAL. */
+/* The configuration a plan matches with (chosen at creation as
+ * cashash_match_plan says).  Errors: EINVAL. */
 int cashash_plan_get_tuning(const cashash_plan* plan, cashash_tuning* out);
 
 /* Forces a configuration (fields normalised to supported values; the plan's
@@ -402,7 +403,8 @@ typedef struct {
   uint64_t n_reevaluated;     /* projections re-evaluated in double (|approx| under the bound) */
   uint64_t n_pairs;           /* pairs in the last match */
   uint64_t n_matches;         /* matches found by the last match */
-  uint64_t n_work_items;      /* (pair, query tile) items of the last match */
+  uint64_t n_work_items;      /* (pair, query tile) items of the last match (0 with the warp-per-query
+                                 kernel, which has none) */
   uint64_t n_launches;        /* kernels launched by this context since it was created */
   double ms_stage[CASHASH_N_STAGES];  /* with profiling on: device milliseconds of each stage of
                                          the last build/match (CUDA events recorded on the
@@ -441,9 +443,10 @@ typedef struct {
   uint32_t n_hyp;        /* 256: at most this many RANSAC hypotheses per pair (1..CASHASH_GA_MAX_HYP) */
   uint32_t inlier_num;   /* 2 */
   uint32_t inlier_den;   /* 3: accepted when inlier_den * inliers >= inlier_num * matches */
-  uint32_t kernel;       /* 0: matching kernel of the subsets chosen by their size (the per-query
-                            kernel when the mean subset image has fewer than 4096 features, else
-                            the join); CASHASH_KERNEL_JOIN / CASHASH_KERNEL_QUERY force one */
+  uint32_t kernel;       /* 0: matching kernel of the subsets chosen by their size (a plan that takes
+                            a warp per query by default keeps it; else the per-query kernel when
+                            the mean subset image has fewer than 4096 features, else the join);
+                            CASHASH_KERNEL_JOIN / CASHASH_KERNEL_QUERY force one */
   double thresh_px;      /* 3.0: inlier when the Sampson distance is <= thresh_px pixels */
   double confidence;     /* 0.99: hypotheses run in batches of 32; after a batch RANSAC stops when
                             (1 - w^8)^N <= 1 - confidence (Hartley and Zisserman, Algorithm 4.5;

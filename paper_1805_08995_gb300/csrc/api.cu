@@ -767,7 +767,10 @@ int plan_configure(cashash_plan* pl, cashash_tuning t) {
 // Plans of at most three pairs take a warp per query by default: even clusters of 8 CTAs leave the join 24 of 304,
 // and its pass has a calibration and a fallback.  us per pass, join / warps: 1 pair of 1,000 x 1,000 features
 // 56 / 12, 8,000 160 / 35, 20,000 520 / 93, 40,000 1,523 / 261; 5-bit short codes 8,000 886 / 80; 3 pairs of 1,000
-// 57 / 14, 4,000 86 / 31.  (Images past 65,535 features, whose tables another kernel builds, were not measured.)
+// 57 / 14, 4,000 86 / 31.  (Images past 65,535 features, whose tables another kernel builds, were not measured.)  Only
+// where the join applies: query images past its limit stay with the per-query kernel, which has the better of short
+// codes there: per-query / warps 52,000 x 52,000, 8 bits 583 / 409, 3 pairs 1,065 / 1,077, with 5 bits 4,509 / 6,178;
+// 65,535, 4 bits 4,731 / 5,975.
 constexpr uint32_t FEW_PAIRS = 3, FEW_FEATURES = 65535;
 bool plan_few(const cashash_plan* pl) {
   if (pl->P == 0 || pl->P > FEW_PAIRS) return false;

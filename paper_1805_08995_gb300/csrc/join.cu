@@ -16,7 +16,12 @@
 // register.  Then the CTA finalises the pair's queries (join_common.cuh).  A
 // query whose list overflowed, or that holds fewer than k distinct survivors
 // while the guess turned some candidate away, is left PENDING for the exact
-// fallback kernel, so results never depend on the guess.
+// fallback kernel, so results never depend on the guess.  A list counts as
+// overflowed once fewer than four of its slots are left and its query meets
+// further candidates: a step takes four of them without a test per store.  Filled
+// to the last slot instead, us per pass over 400 pairs of 6,000 x 6,000 features: 8
+// bits, k = 2 892 -> 917, 6 tables of 4 bits, k = 2 5,215 -> 5,476, k = 16 26,369 ->
+// 24,673.
 //
 // With the band (EPI) a candidate outside it is no candidate at all, so there is
 // no Hamming guess, and the band test, cheaper than a Hamming distance and passed
@@ -28,7 +33,7 @@
 // each survivor out of the accumulator layout cost more instructions than the
 // counts they replace.  Per lookup entry (500 pairs of 8k x 8k features): 2.40
 // warp instructions with FP8 mma.sync in 16 x 32 blocks (35 % of their slots were
-// entries), 1.59 here.  f16 operands that hold two code bits each (four MMAs per
+// entries), 1.60 here.  f16 operands that hold two code bits each (four MMAs per
 // 16 x 8 tile, exact in f32 accumulators) took 20.6 ms on the 4,950 pairs below.
 // What bounds the kernel now is memory latency and issue (56 % of the slots; half
 // of the stalls wait for tables, lists and rows): with two CTAs of 512 threads
@@ -502,7 +507,9 @@ uint32_t join_lg(uint32_t n_items, int nsm) {
 
 uint32_t join_grid(const KParams& kp, uint32_t na_max, uint32_t n_items, uint32_t ctas_per_sm) {
   const bool epi = kp.epi_px >= 0.0;
-  // query images whose 32-bit counters and keys would exceed a CTA's shared memory take the per-query kernel
+  // The largest query image: what 32-bit counters of a CTA of JT threads leave room for (k_join_tc's limit, and what
+  // the plans' kernel rules were measured with); above it the per-query kernel.  Counters of a byte would let this
+  // kernel take more; larger images were not measured with it.
   if ((size_t)4 * ((na_max + 3) / 4 * 4) + (size_t)2 * join_kc(kp.top_k) * JT * 4 + 4096 > 227u * 1024u) return 0;
   int dev = 0, nsm = 0, ncl = 0;
   cudaGetDevice(&dev);
