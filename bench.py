@@ -72,13 +72,14 @@ def peaks():
 
 def workload(name: str, rank: int, precision: str = "bf16"):
     """The synthetic image set of a named workload and its description.  On
-    the 100-image exhaustive set the plain FP32 projection is config 1 and the
-    BF16 tensor-core projection (with exact re-evaluation) is config 2."""
+    the 100-image exhaustive set the FP32 setting is config 1 and the BF16
+    setting config 2 (one projection, with exact re-evaluation, for both)."""
     import synth
     if name == "config1":
         s = synth.config1(seed=1 + 1000 * rank)
-        tag = ("config2: BF16 tensor-core projection (exact FP64 re-evaluation under its bound) on the config-1 set"
-               if precision == "bf16" else "config1: plain FP32 projection")
+        tag = ("config2: BF16 setting (tensor-core projection with R in three f16 terms, exact FP64 re-evaluation "
+               "under its bound) on the config-1 set" if precision == "bf16" else "config1: FP32 setting (the same "
+               "projection)")
         desc = tag + ": 100 images x U{4000..12000} SIFT-like uint8 descriptors (30%% noisy copies of " \
                "index-neighbours), all 4950 pairs, seed %d" % (1 + 1000 * rank)
     elif name == "config0":
@@ -578,7 +579,7 @@ def run_ours(args):
         line = {"metric": METRIC, "value": value, "unit": "pairs/s", "n_gpus": world, "steps": args.steps,
                 "warmup": args.warmup, "ms_per_step": t_max * 1e3 / args.steps, "higher_is_better": True,
                 "scaling": "strong" if split_pairs else "weak", "vs_baseline": None,
-                "dtype": "u8/" + ("bf16" if prec == ch.CASHASH_BF16 else "fp32") + "+f64fix",
+                "dtype": "u8/f16x3+f64fix",
                 "data": "synthetic",
                 "config": {"workload": wdesc, "images": int(s.n_images), "features": int(s.desc.shape[0]),
                            "pairs": P_job if split_pairs else P, "precision": args.precision,
@@ -619,7 +620,7 @@ def config3_forms(ch, torch, dev):
     """Config 3 (2,000 images, 59,556 pairs) in the two forms its target
     compares: the batched BF16 form (one persistent launch per step over the
     device pair list, CUDA-graph captured, autotuned on a sample of pairs) and
-    the plain FP32 form with one launch per pair.  Device time per step with
+    the FP32 form with one launch per pair.  Device time per step with
     CUDA events, L2 flushed before each step."""
     import synth
     s = synth.config3()
@@ -741,7 +742,7 @@ def run_tau_sweep(args):
         r["recall_vs_tau128"] = r["recall"] / base["recall"] if base else None
         r["speed_vs_tau128"] = r["pairs_per_s"] / base["pairs_per_s"] if base else None
     line = {"metric": METRIC, "unit": "pairs/s", "n_gpus": 1, "steps": args.steps, "warmup": args.warmup,
-            "higher_is_better": True, "data": "synthetic", "dtype": "u8/bf16+f64fix",
+            "higher_is_better": True, "data": "synthetic", "dtype": "u8/f16x3+f64fix",
             "config": {"workload": wdesc, "l2": "flushed: 256 MiB write before every timed step",
                        "recall_def": "planted noisy-copy correspondences found among the matches"},
             "tau_sweep": rows, "clocks": clocks}
@@ -919,7 +920,7 @@ def run_ga(args):
         cpu = {"value": v, "unit": "pairs/s", "cores": cores, "kind": "oracle", "sample": text, "seconds": secs}
     line = {"metric": METRIC, "value": P / t_step, "unit": "pairs/s", "n_gpus": 1, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": t_step * 1e3, "higher_is_better": True, "scaling": "weak",
-            "vs_baseline": None, "dtype": "u8/bf16+f64fix, f64 geometry", "data": "synthetic",
+            "vs_baseline": None, "dtype": "u8/f16x3+f64fix, f64 geometry", "data": "synthetic",
             "config": {"workload": wdesc.replace("ground-truth F", "F estimated by the first stage (Ga-CasHash)"),
                        "pairs": P, "features": int(s.desc.shape[0]),
                        "ga": {"stage1_kernel": args.ga_kernel, "confidence": gp.confidence, "top_pct": gp.top_pct, "min_matches": gp.min_matches, "n_hyp": gp.n_hyp,
