@@ -265,6 +265,7 @@ cudaError_t launch_build_tables(const uint8_t* buckets, const uint32_t* codes, c
                                 const uint64_t* chunk_f0, const uint32_t* chunk_len, uint32_t n_chunks,
                                 uint32_t n_tables, uint8_t* tables, cudaStream_t s);
 bool tables_one_launch(uint32_t n_max);
+int tables_warps(uint32_t n_max, uint64_t tasks, int nsm);  // warps of a sorting CTA
 
 struct MatchArgs {
   const uint8_t* desc;

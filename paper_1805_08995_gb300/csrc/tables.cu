@@ -29,8 +29,8 @@ namespace chx {
 // in one launch; 321,454: 176, 159, 151; 4,000: 40.4, 39.6, 35.1.  What is left waits
 // for the gathered codes and for shared memory.
 constexpr uint32_t BJ_MAX_N = 65535;  // local indices held as uint16 in shared memory
-constexpr int NW = 16;                // warps of a CTA (8 or 32: within 1 %; one pair 2 us slower with 8)
 
+template <int NW>
 __global__ void __launch_bounds__(NW * 32) k_sort_tables(const uint8_t* __restrict__ buckets,
                                                          const uint32_t* __restrict__ codes,
                                                          const uint64_t* __restrict__ img_f0,
@@ -139,7 +139,13 @@ __global__ void __launch_bounds__(NW * 32) k_sort_tables(const uint8_t* __restri
   }
 }
 
-static size_t sort_smem(uint32_t n_max) { return NW * 256 * 4 + (size_t)(n_max + 7) / 8 * 8 * 3; }
+// Warps of a CTA: 8 where images are small and their CTAs more than the SMs, else 16.  A CTA clears and adds up a
+// histogram per warp whatever it sorts, and twice the CTAs fit an SM; few CTAs, and large images, gain from the
+// warps.  us a build with 8 / 16 (6 tables): 2,000 images of 64 features 138 / 209, 256 234 / 308, 1,000 of 1,000 341 /
+// 373, 200 of 4,000 276 / 282, 100 of 8,000 288 / 281, 2 of 1,000 39.6 / 37.3, 2 of 4,000 45.4 / 43.6.
+int tables_warps(uint32_t n_max, uint64_t tasks, int nsm) { return n_max <= 4096 && tasks > (uint64_t)nsm ? 8 : 16; }
+
+static size_t sort_smem(uint32_t n_max, int nw) { return nw * 256 * 4 + (size_t)(n_max + 7) / 8 * 8 * 3; }
 
 // Join tables of a set with an image of more than BJ_MAX_N features: one warp
 // per (image, table), a stable counting sort over the whole image with global
@@ -211,7 +217,7 @@ __global__ void __launch_bounds__(256) k_build_join(const uint8_t* __restrict__ 
 // Image and chunk tables in one launch while the images' shared memory leaves room for four CTAs of an SM, as many
 // as its threads do (up to 13,640 features); else the chunks would run fewer at a time than they can.  An SM has 228
 // KB, of which the system takes 1 KB for each CTA and the kernel's static arrays 32 bytes.
-bool tables_one_launch(uint32_t n_max) { return sort_smem(n_max) <= 228 * 1024 / 4 - 1024 - 32; }
+bool tables_one_launch(uint32_t n_max) { return sort_smem(n_max, 16) <= 228 * 1024 / 4 - 1024 - 32; }
 
 cudaError_t launch_build_tables(const uint8_t* buckets, const uint32_t* codes, const uint64_t* img_f0,
                                 const uint32_t* img_n, const uint64_t* img_join, uint32_t n_images, uint32_t n_max,
@@ -222,18 +228,21 @@ cudaError_t launch_build_tables(const uint8_t* buckets, const uint32_t* codes, c
     return cudaErrorInvalidValue;  // one CTA (or warp) per image or chunk and table
   static_assert(JC <= (int)BJ_MAX_N, "chunk tables sort in shared memory");
   static int attr_dev = -1;
-  int dev = 0;
+  int dev = 0, nsm = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  if (attr_dev != dev) {
-    e = cudaFuncSetAttribute(k_sort_tables, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sort_smem(BJ_MAX_N));
+  if (attr_dev != dev) {  // (8 warps: at most 20 KB)
+    e = cudaFuncSetAttribute(k_sort_tables<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sort_smem(BJ_MAX_N, 16));
     if (e != cudaSuccess) return e;
     attr_dev = dev;
   }
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   auto sort = [&](uint64_t join_tasks, uint64_t tasks, uint32_t n) {
     if (tasks == 0) return cudaSuccess;
-    k_sort_tables<<<(unsigned)tasks, NW * 32, sort_smem(n), s>>>(buckets, codes, img_f0, img_n, img_join, chunk_f0,
-                                                                 chunk_len, n_tables, (uint32_t)join_tasks, tables);
+    const int nw = tables_warps(n_max, tasks, nsm);
+    (nw == 8 ? k_sort_tables<8> : k_sort_tables<16>)<<<(unsigned)tasks, nw * 32, sort_smem(n, nw), s>>>(
+        buckets, codes, img_f0, img_n, img_join, chunk_f0, chunk_len, n_tables, (uint32_t)join_tasks, tables);
     return cudaGetLastError();
   };
   if (tables_one_launch(n_max)) return sort(jt, jt + ct, n_max);
