@@ -40,7 +40,7 @@ L2_FLUSH_BYTES = 256 << 20
 # summarised in profiles/ (valid only for the kernel source it was taken on).
 PROFILED_TRAFFIC = {
     "k_join": {"sources": ["paper_1805_08995_gb300/csrc/join.cu", "paper_1805_08995_gb300/csrc/join_common.cuh"],
-               "sha256": "bc959682463f088e833c52c52168835c0f8e7d59d4b0c6b6fab1c797bcea23a0",
+               "sha256": "b14cee04e3a3cd87ccb13dae32f5592b4533d546d12f1831d84b05967eeaae77",
                "bytes_per_entry": (2.498390e9 + 1.100804e9) / 861951265},
 }
 

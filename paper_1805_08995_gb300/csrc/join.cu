@@ -39,8 +39,8 @@
 // of the stalls wait for tables, lists and rows): with two CTAs of 512 threads
 // per SM the lists of the pairs in flight (about 1.2 MB each) exceed the L2 (a
 // timing copy whose lists fit it: 8.9 ms instead of 14 for the scan).  4,950
-// pairs of 8k x 8k: 25.0 -> 16.7 ms; 11,527 uneven pairs (1,000 to 20,000
-// features): 52.9 -> 31.3 ms.
+// pairs of 8k x 8k: 25.0 -> 16.8 ms; 11,527 uneven pairs (1,000 to 20,000
+// features): 52.9 -> 31.6 ms.
 #include <cooperative_groups.h>
 
 #include "join_common.cuh"
